@@ -115,6 +115,8 @@ def step_kernel_of(w, variant="auto"):
             w["dtype"] in ("F16S", "BF16S") or (w["dtype"] == "F32" and w["q"] == 9
                                                  and cells >= 1 << 17)):
         return pair
+    if w["dtype"] == "F64":
+        return "fused_step_f64_kernel", ("lbm_step_f64.cuh", "lbm_step.cuh", "lbm_traits.cuh")
     return "fused_step_kernel", ("lbm_step.cuh", "lbm_traits.cuh")
 
 

@@ -233,7 +233,7 @@ __device__ __forceinline__ float rcp_approx(float x) {
     return r;
 }
 
-// Moments, equilibrium, sensor and BGK collision of one cell from its gathered deviations df;
+// Moments, equilibrium, sensor and BGK collision of one cell in FP32 from its gathered deviations df;
 // emit(i, d) receives the post-collision deviation d = f*_i - w_i of every population.  Returns
 // the sensor K (MODE != 0).
 template <class L, int DT, int MODE, class Emit>
@@ -267,13 +267,8 @@ __device__ __forceinline__ typename Storage<DT>::R relax_cell(const typename Sto
         const R dfeq = w * (drho + rho * P);  // f^eq_i - w_i
         const R fneq = df[i] - dfeq;
         if (MODE != 0) {
-            if constexpr (sizeof(R) == 4) {
-                // f^eq_i = (f^eq_i - w_i) + w_i: one add, one reciprocal, one fused multiply-add
-                ksum = fmaf(fabsf(fneq), rcp_approx(dfeq + w), ksum);
-            } else {
-                const R feq = w * rho * (R(1) + P);
-                ksum += fabs(fneq) / feq;
-            }
+            // f^eq_i = (f^eq_i - w_i) + w_i: one add, one reciprocal, one fused multiply-add
+            ksum = fmaf(fabsf(fneq), rcp_approx(dfeq + w), ksum);
         }
         emit(i, df[i] - omega * fneq);
     }

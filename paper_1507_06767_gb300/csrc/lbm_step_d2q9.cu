@@ -1,6 +1,7 @@
 // D2Q9 instantiations of the fused step: the one-cell kernel (lbm_step.cuh) and the two-cell packed
 // kernel (lbm_step_pair.cuh), with the automatic choice between them.
 #include "lbm_internal.h"
+#include "lbm_step_f64.cuh"
 #include "lbm_step_pair.cuh"
 
 namespace lbm {
@@ -20,7 +21,7 @@ cudaError_t step_d2q9(int dtype, const void *fin, void *fout, const StepParams &
     if (has_halo(p)) {
         if (variant != KERNEL_AUTO && variant != KERNEL_CELL) return cudaErrorInvalidValue;
         switch (dtype) {
-            case 0: return launch_fused_step<D2Q9, 0, true>(fin, fout, p, mode, tile_max, k_field, s);
+            case 0: return launch_fused_step_f64<D2Q9, true>(fin, fout, p, mode, tile_max, k_field, s);
             case 1: return launch_fused_step<D2Q9, 1, true>(fin, fout, p, mode, tile_max, k_field, s);
             case 2: return launch_fused_step<D2Q9, 2, true>(fin, fout, p, mode, tile_max, k_field, s);
             case 3: return launch_fused_step<D2Q9, 3, true>(fin, fout, p, mode, tile_max, k_field, s);
@@ -28,7 +29,7 @@ cudaError_t step_d2q9(int dtype, const void *fin, void *fout, const StepParams &
         }
     }
     switch (dtype) {
-        case 0: return launch_fused_step<D2Q9, 0>(fin, fout, p, mode, tile_max, k_field, s);
+        case 0: return launch_fused_step_f64<D2Q9>(fin, fout, p, mode, tile_max, k_field, s);
         case 1:
             return pair ? launch_fused_step_pair<D2Q9, 1>(fin, fout, p, mode, tile_max, k_field, s)
                         : launch_fused_step<D2Q9, 1>(fin, fout, p, mode, tile_max, k_field, s);

@@ -6,6 +6,7 @@
 #include <mutex>
 
 #include "lbm_internal.h"
+#include "lbm_step_f64.cuh"
 #include "lbm_step_pair.cuh"
 #include "lbm_step_tma.cuh"
 #include "lbm_step_tma_pair.cuh"
@@ -186,7 +187,7 @@ cudaError_t step_d3q19(int dtype, const void *fin, void *fout, const StepParams 
     if (has_halo(p)) {  // a slab with cut faces: the one-cell kernel with the halo gather
         if (variant != KERNEL_AUTO && variant != KERNEL_CELL) return cudaErrorInvalidValue;
         switch (dtype) {
-            case 0: return launch_fused_step<D3Q19, 0, true>(fin, fout, p, mode, tile_max, k_field, s);
+            case 0: return launch_fused_step_f64<D3Q19, true>(fin, fout, p, mode, tile_max, k_field, s);
             case 1: return launch_fused_step<D3Q19, 1, true>(fin, fout, p, mode, tile_max, k_field, s);
             case 2: return launch_fused_step<D3Q19, 2, true>(fin, fout, p, mode, tile_max, k_field, s);
             case 3: return launch_fused_step<D3Q19, 3, true>(fin, fout, p, mode, tile_max, k_field, s);
@@ -198,7 +199,7 @@ cudaError_t step_d3q19(int dtype, const void *fin, void *fout, const StepParams 
         return launch_fused_step_tma_pair<3>(fin, fout, p, mode, tile_max, k_field, s);
     }
     switch (dtype) {
-        case 0: return launch_fused_step<D3Q19, 0>(fin, fout, p, mode, tile_max, k_field, s);
+        case 0: return launch_fused_step_f64<D3Q19>(fin, fout, p, mode, tile_max, k_field, s);
         case 1:
             if (tma) return launch_fused_step_tma<1>(fin, fout, p, mode, tile_max, k_field, s);
             return pair ? launch_fused_step_pair<D3Q19, 1>(fin, fout, p, mode, tile_max, k_field, s)
