@@ -15,7 +15,7 @@
 // without cancelling against w_i.
 #pragma once
 
-#include "lbm_traits.cuh"
+#include "lbm_internal.h"
 
 namespace lbm {
 
@@ -311,6 +311,8 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, LBM_STEP_MIN_BLOCKS)
     const size_t N = (size_t)nx * ny * nz;
     const R omega = param_omega<R>(p);
 
+    if constexpr (L::D == 2) fin = pdl_wait(fin);
+
     // clear the other tile buffer for the next sensor step (kernels that combine tiles across
     // CTAs with atomics need it zeroed)
     if (MODE != 0 && p.tile_zero) {
@@ -373,6 +375,17 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, LBM_STEP_MIN_BLOCKS)
     }
 }
 
+// Launch of a step kernel.  In 2-D, where a step may take a few us, it overlaps its start with the
+// end of the step before (launch_pdl): 128^2 FP64 4.95 -> 4.80 us a step.  In 3-D the CTAs that wait
+// take the place of running ones: 195 x 129 x 97 FP32 78.0 -> 79.7 us, so not there.
+template <class L, class... Params, class... Args>
+inline cudaError_t launch_step_kernel(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem,
+                                      cudaStream_t s, Args... args) {
+    if (L::D == 2) return launch_pdl(kernel, grid, block, smem, s, args...);
+    kernel<<<grid, block, smem, s>>>(args...);
+    return cudaGetLastError();
+}
+
 template <class L, int DT, bool HALO = false>
 cudaError_t launch_fused_step(const void *fin, void *fout, const StepParams &p, int mode,
                               void *tile_max, void *k_field, cudaStream_t stream) {
@@ -386,12 +399,10 @@ cudaError_t launch_fused_step(const void *fin, void *fout, const StepParams &p, 
     R *tm = static_cast<R *>(tile_max);
     R *kf = static_cast<R *>(k_field);
     if (mode == 0)
-        fused_step_kernel<L, DT, 0, HALO><<<grid, block, 0, stream>>>(a, b, p, tm, kf);
-    else if (mode == 1)
-        fused_step_kernel<L, DT, 1, HALO><<<grid, block, 0, stream>>>(a, b, p, tm, kf);
-    else
-        fused_step_kernel<L, DT, 2, HALO><<<grid, block, 0, stream>>>(a, b, p, tm, kf);
-    return cudaGetLastError();
+        return launch_step_kernel<L>(fused_step_kernel<L, DT, 0, HALO>, grid, block, 0, stream, a, b, p, tm, kf);
+    if (mode == 1)
+        return launch_step_kernel<L>(fused_step_kernel<L, DT, 1, HALO>, grid, block, 0, stream, a, b, p, tm, kf);
+    return launch_step_kernel<L>(fused_step_kernel<L, DT, 2, HALO>, grid, block, 0, stream, a, b, p, tm, kf);
 }
 
 // A slab with halo faces (StepParams::halo_lo / halo_hi) runs the one-cell kernel with the halo

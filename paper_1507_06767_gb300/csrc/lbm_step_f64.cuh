@@ -146,6 +146,7 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, 2)
     const int x = bx * CTA_X + lane, y = by * blockDim.y + threadIdx.y, z0 = bz * ZT;
     const bool active = (x < nx) && (y < ny);
     const size_t N = (size_t)nx * ny * nz;
+    if constexpr (L::D == 2) fin = pdl_wait(fin);
     if (MODE != 0 && p.tile_zero) {  // as in fused_step_kernel
         const size_t nt = (size_t)p.ntx * p.nty * p.ntz, me = (size_t)blockIdx.x * (CTA_X * CTA_Y) +
                                                               threadIdx.y * CTA_X + lane;
@@ -212,12 +213,10 @@ cudaError_t launch_fused_step_f64(const void *fin, void *fout, const StepParams 
            *kf = static_cast<double *>(k_field);
     const RelaxF64 k(p);
     if (mode == 0)
-        fused_step_f64_kernel<L, 0, HALO><<<grid, block, 0, stream>>>(a, b, p, tm, kf, k);
-    else if (mode == 1)
-        fused_step_f64_kernel<L, 1, HALO><<<grid, block, 0, stream>>>(a, b, p, tm, kf, k);
-    else
-        fused_step_f64_kernel<L, 2, HALO><<<grid, block, 0, stream>>>(a, b, p, tm, kf, k);
-    return cudaGetLastError();
+        return launch_step_kernel<L>(fused_step_f64_kernel<L, 0, HALO>, grid, block, 0, stream, a, b, p, tm, kf, k);
+    if (mode == 1)
+        return launch_step_kernel<L>(fused_step_f64_kernel<L, 1, HALO>, grid, block, 0, stream, a, b, p, tm, kf, k);
+    return launch_step_kernel<L>(fused_step_f64_kernel<L, 2, HALO>, grid, block, 0, stream, a, b, p, tm, kf, k);
 }
 
 }  // namespace lbm

@@ -213,6 +213,7 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, DT == 1 ? LBM_PAIR_MIN_BLOCKS_F3
     const unsigned nxy = (unsigned)nx * (unsigned)ny;
 
     int kmax = 0;
+    if constexpr (L::D == 2) fin = pdl_wait(fin);
 
     if (MODE != 0 && p.tile_zero) {
         const size_t nt = (size_t)p.ntx * p.nty * p.ntz;
@@ -348,12 +349,10 @@ cudaError_t launch_fused_step_pair(const void *fin, void *fout, const StepParams
     float *tm = static_cast<float *>(tile_max);
     float *kf = static_cast<float *>(k_field);
     if (mode == 0)
-        fused_step_pair_kernel<L, DT, 0><<<grid, block, 0, stream>>>(a, b, p, tm, kf);
-    else if (mode == 1)
-        fused_step_pair_kernel<L, DT, 1><<<grid, block, 0, stream>>>(a, b, p, tm, kf);
-    else
-        fused_step_pair_kernel<L, DT, 2><<<grid, block, 0, stream>>>(a, b, p, tm, kf);
-    return cudaGetLastError();
+        return launch_step_kernel<L>(fused_step_pair_kernel<L, DT, 0>, grid, block, 0, stream, a, b, p, tm, kf);
+    if (mode == 1)
+        return launch_step_kernel<L>(fused_step_pair_kernel<L, DT, 1>, grid, block, 0, stream, a, b, p, tm, kf);
+    return launch_step_kernel<L>(fused_step_pair_kernel<L, DT, 2>, grid, block, 0, stream, a, b, p, tm, kf);
 }
 
 }  // namespace lbm

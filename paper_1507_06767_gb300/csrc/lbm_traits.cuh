@@ -122,6 +122,22 @@ struct Bits<double> {
     using type = long long;
 };
 
+// Wait until the launch before this one (launch_pdl) has ended and its writes are visible, then let
+// the next one start.  The pointer comes back through the wait: loads from it, also those of the
+// read-only path, which the compiler may otherwise move, cannot go ahead of it.
+template <class T>
+__device__ __forceinline__ T *pdl_wait(T *p) {
+    asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" : "+l"(p) : : "memory");
+    return p;
+}
+
+// Another pointer that is read after pdl_wait: it is not known before the wait.
+template <class T>
+__device__ __forceinline__ T *pdl_order(T *p) {
+    asm volatile("" : "+l"(p) : : "memory");
+    return p;
+}
+
 struct StepParams {
     int nx, ny, nz;
     int periodic;      // bit 0 x, bit 1 y, bit 2 z

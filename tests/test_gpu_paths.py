@@ -30,3 +30,29 @@ def test_fp64_pairwise_relaxation(L, q, dims, periodic, scale):  # noqa: F811
     assert rel(lat.populations(), f) <= 1e-14
     assert rel(lat.sensor_field(), K) <= 1e-12
     lat.close()
+
+
+@pytest.mark.parametrize("dtype", ["LBM_F64", "LBM_F32", "LBM_BF16S"])
+@pytest.mark.parametrize("dims,periodic", [((33, 17), 0), ((128, 128), 1), ((700, 302), 2)])
+def test_2d_runs_in_graphs_have_the_bits_of_single_steps(L, dims, periodic, dtype):  # noqa: F811
+    """A 2-D step's CTAs may start before the step before it has ended: runs of them in graphs, and
+    with sensor steps and reads between, must give what steps with a wait after each give."""
+    o = O.Oracle(9, *dims, 1, tau=0.7, lid=(0.1, 0.0, 0.0), periodic=periodic)
+    f = perturbed(o, seed=5 + sum(dims), amp=0.02)
+    import torch
+
+    lats = [L.Lattice(9, *dims, 1, 0.7, dtype=getattr(L, dtype), lid=(0.1, 0.0), periodic=periodic)
+            for _ in range(2)]
+    for lat in lats:
+        lat.set_populations(f)
+        L.lbm_set_sensor_every(lat.h, 37)
+    L.lbm_set_graphs(lats[1].h, 0)
+    for n in (40, 100):
+        lats[0].step(n)
+        for _ in range(n):
+            lats[1].step(1)
+            torch.cuda.synchronize()
+        assert np.array_equal(lats[0].raw(), lats[1].raw())
+        assert np.array_equal(lats[0].sensor(8), lats[1].sensor(8))
+    for lat in lats:
+        lat.close()
