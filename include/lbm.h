@@ -567,6 +567,10 @@ LBM_API int lbm_regrid(lbm_t *h, const double *field_dev, const lbm_regrid_param
  * e.g. with gradients averaged over several processes); lbm_net_train_step is backward + Adam
  * (beta1 0.9, beta2 0.999, eps 1e-8).  A non-NULL loss_host receives the loss and synchronises;
  * otherwise the calls queue their kernels on the network's stream (lbm_net_set_stream) and return.
+ * lbm_net_train_epoch takes `steps` such steps, step s on the minibatch of the `batch` rows
+ * idx_dev[s * batch ...] of the training set (nrows items of x_dev and of target_dev), queued one
+ * behind the other; it returns when they are done, losses_host (may be NULL) holding the loss of
+ * each.  An index outside [0, nrows) is not read and gives LBM_EINVAL at the end.
  * lbm_net_set_params sets the parameters and clears the Adam state.  Targets and predictions are
  * in log10 units: lbm_net_log_targets writes t = log10(max(K, floor_k)) - offset for n block
  * maxima (NaN for a NaN maximum), lbm_net_to_maxima K = 10^(y + offset); the latter feeds lbm_flags_from_maxima.
@@ -588,6 +592,9 @@ LBM_API int lbm_net_backward(lbm_net *n, const float *x_dev, const float *target
 LBM_API int lbm_net_adam(lbm_net *n, float lr, float beta1, float beta2, float eps);
 LBM_API int lbm_net_train_step(lbm_net *n, const float *x_dev, const float *target_dev, int batch,
                                int h, int w, float lr, double *loss_host);
+LBM_API int lbm_net_train_epoch(lbm_net *n, const float *x_dev, const float *target_dev,
+                                long long nrows, const int *idx_dev, int steps, int batch, int h,
+                                int w, float lr, double *losses_host);
 LBM_API int lbm_net_log_targets(const double *kmax_dev, long long n, float offset, float floor_k,
                                 float *t_dev, void *stream);
 /*

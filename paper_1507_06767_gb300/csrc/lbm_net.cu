@@ -9,9 +9,11 @@
 // x 9 weights), so each kernel keeps its weights in shared memory and works on a staged tile of
 // pixels; sums over pixels are added in a fixed order, so a training step is deterministic.
 //
-// A training step of 16 x 64 x 64 pixels (1.1 GFLOP, 16 us at the FP32 rate) takes 139 us on the
-// device and host with its minibatch gather and loss readback, 780 us before the kernels were
-// tiled: the weight gradients took 960 us of 1080 us of serialised kernel time, now 30 us of 91.
+// A training step of 16 x 64 x 64 pixels (1.1 GFLOP, 16 us at the FP32 rate) takes 106 us in an
+// epoch, 780 us before the kernels were tiled (the weight gradients took 960 us of 1080 us of
+// serialised kernel time, now 30 us of 84) and 144 us while each step gathered its minibatch in two
+// launches and the host waited for its loss.  The launches overlap their starts with the end of the
+// one before (launch_pdl).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -206,17 +208,36 @@ __device__ __forceinline__ void store_px(float *p, const float (&v)[PX], int n, 
         if (k < n) p[k] = v[k];
 }
 
+// Where the items of a minibatch lie in the training set: item b is row idx[b] of nrows, or row b
+// without idx.  An index outside the set sets *bad and reads row 0.
+struct Rows {
+    const int *idx;
+    long long nrows;
+    int *bad;
+    __device__ __forceinline__ int of(int b) const {
+        if (!idx) return b;
+        const int r = idx[b];
+        if (r >= 0 && r < nrows) return r;
+        *bad = 1;
+        return 0;
+    }
+};
+
 // out[b, o, y, x] = relu(bias[o] + sum_{c,i,j} W[o, c, i, j] in[b, c, y+i-1, x+j-1]).  FIRST: the
 // input is the caller's FP32 field, normalised and rounded to BF16 as it is staged (and kept in x0,
 // which the weight gradient reads); else BF16 activations.  2 x TILE_Y x COUT threads.  At 16 x 64
 // x 64, 16 -> 16 channels: 28.2 -> 12.1 us against one pixel a thread; 4 -> 16 with the
-// normalisation: 10.0 + 5.4 -> 6.7 us.
+// normalisation: 10.0 + 5.4 -> 6.7 us.  FIRST takes its items where `rows` says, so a minibatch needs
+// no gather of its own.
 template <int CIN, int COUT, bool FIRST>
 __global__ void __launch_bounds__(TILE_QUADS *TILE_Y *(COUT / 4))
     k_conv_relu(const void *__restrict__ in, const Norm nm, bf16 *__restrict__ x0_out,
                 const float *__restrict__ W, const bf16 *__restrict__ bias, const Tiling g,
-                bf16 *__restrict__ out) {
+                bf16 *__restrict__ out, const Rows rows) {
     constexpr int THREADS = TILE_QUADS * TILE_Y * (COUT / 4);
+    in = pdl_wait(in);
+    W = pdl_order(W);
+    bias = pdl_order(bias);
     constexpr int PITCH = (TILE_Y + 2) * ROW_PITCH;
     __shared__ __align__(16) float ws[CIN * 9 * COUT];
     __shared__ __align__(16) float xs[CIN * PITCH];
@@ -225,7 +246,7 @@ __global__ void __launch_bounds__(TILE_QUADS *TILE_Y *(COUT / 4))
     stage_weights<CIN * 9 * COUT, THREADS>(W, ws);  // [c][tap][o]
     if constexpr (FIRST) {
         stage_window<CIN, TILE_Y, THREADS>(
-            static_cast<const float *>(in), b, y0, x0, g, xs, PITCH,
+            static_cast<const float *>(in), rows.of(b), y0, x0, g, xs, PITCH,
             [&](int c, float v) {
                 return __bfloat162float(__float2bfloat16_rn((v - nm.shift[c]) * nm.scale[c]));
             });
@@ -280,13 +301,17 @@ __global__ void __launch_bounds__(TILE_QUADS *TILE_Y *(COUT / 4))
 // order, so the sums are deterministic.
 constexpr int OUT_GROUPS = 4;
 constexpr int OUT_THREADS = TILE_QUADS * TILE_Y * OUT_GROUPS;
+constexpr int LOSS_SLOTS = 1024;  // steps queued at most before the host reads their losses
 constexpr int LOSS_PARTS = 512;  // CTAs of the output layer at most, one partial sum each
 
 template <int CIN, bool GRAD>
 __global__ void __launch_bounds__(OUT_THREADS)
     k_conv_out(const bf16 *__restrict__ in, const bf16 *__restrict__ W, const bf16 *__restrict__ bias,
                const Tiling g, long long tiles, float *__restrict__ out, const float *__restrict__ t,
-               float two_n, float *__restrict__ dy, double *__restrict__ loss_part) {
+               float two_n, float *__restrict__ dy, double *__restrict__ loss_part, const Rows rows) {
+    in = pdl_wait(in);
+    W = pdl_order(W);
+    bias = pdl_order(bias);
     static_assert(CIN % OUT_GROUPS == 0 && OUT_THREADS == TILE_X * TILE_Y, "unsupported layer shape");
     constexpr int PITCH = (TILE_Y + 2) * ROW_PITCH, CPT = CIN / OUT_GROUPS;
     __shared__ __align__(16) float xs[CIN * PITCH];
@@ -333,7 +358,7 @@ __global__ void __launch_bounds__(OUT_THREADS)
             const size_t at = ((size_t)b * g.H + y) * g.W + x;
             out[at] = v;
             if (GRAD) {
-                const float d = v - t[at];
+                const float d = v - t[((size_t)rows.of(b) * g.H + y) * g.W + x];
                 dy[at] = two_n * d;
                 loss += (double)d * (double)d;
             }
@@ -359,6 +384,9 @@ template <int CIN, int COUT>
 __global__ void __launch_bounds__(TILE_QUADS *TILE_Y *(CIN / 4))
     k_conv_bwd_data(const float *__restrict__ dO, const float *__restrict__ W,
                     const bf16 *__restrict__ A, const Tiling g, float *__restrict__ dA) {
+    dO = pdl_wait(dO);
+    W = pdl_order(W);
+    A = pdl_order(A);
     constexpr int THREADS = TILE_QUADS * TILE_Y * (CIN / 4);
     constexpr int PITCH = (TILE_Y + 2) * ROW_PITCH;
     __shared__ __align__(16) float ws[COUT * 9 * CIN];
@@ -521,8 +549,14 @@ struct WgradArgs {
     long long tiles;
 };
 template <int CI, int HD>
-__global__ void __launch_bounds__(WG_THREADS) k_wgrad(const WgradArgs a, const Tiling g) {
+__global__ void __launch_bounds__(WG_THREADS) k_wgrad(WgradArgs a, const Tiling g) {
     extern __shared__ __align__(16) float sm[];
+    a.dy = pdl_wait(a.dy);
+    a.dz2 = pdl_order(a.dz2);
+    a.dz1 = pdl_order(a.dz1);
+    a.a2 = pdl_order(a.a2);
+    a.a1 = pdl_order(a.a1);
+    a.x0 = pdl_order(a.x0);
     int k = blockIdx.x;
     if (k < a.ctas[1]) {
         conv_bwd_weight<HD, HD>(a.dz2, a.a1, g, a.tiles, k, a.ctas[1], sm, a.part[1]);
@@ -587,7 +621,8 @@ struct ReduceArgs {
 };
 constexpr int RED_PARAMS = 32, RED_SLICES = 16;
 __global__ void __launch_bounds__(RED_PARAMS *RED_SLICES)
-    k_net_reduce(const ReduceArgs r, const AdamArgs a) {
+    k_net_reduce(ReduceArgs r, const AdamArgs a) {
+    r.loss_part = pdl_wait(r.loss_part);
     __shared__ float sh[RED_SLICES][RED_PARAMS];
     __shared__ double shl[RED_SLICES];
     const int lane = threadIdx.x % RED_PARAMS, slice = threadIdx.x / RED_PARAMS;
@@ -609,7 +644,7 @@ __global__ void __launch_bounds__(RED_PARAMS *RED_SLICES)
     if (p < r.nparam) {
         int l = 0, q = p;
         while (q >= r.count[l]) q -= r.count[l++];
-        const float *src = r.part[l] + q;
+        const float *src = pdl_order(r.part[l]) + q;
         const size_t pitch = r.count[l];
         const int per = (r.ctas[l] + RED_SLICES - 1) / RED_SLICES, k0 = slice * per;
         const int k1 = min(k0 + per, r.ctas[l]);
@@ -769,7 +804,8 @@ struct lbm_net_s {
     __nv_bfloat16 *x0 = nullptr, *a1 = nullptr, *a2 = nullptr;
     float *y = nullptr, *dy = nullptr, *dz1 = nullptr, *dz2 = nullptr;
     double *loss_part = nullptr;
-    double *loss_host = nullptr, *loss_dev = nullptr;  // pinned host memory and its device address
+    // pinned host memory and its device address: the losses of up to LOSS_SLOTS steps, an error word
+    double *loss_host = nullptr, *loss_dev = nullptr;
     float *wpart[3] = {nullptr, nullptr, nullptr};  // partial weight gradients of the layers
     long long last_pos = 0;  // positions of the last forward / backward call (0: none yet)
 };
@@ -840,40 +876,46 @@ int out_ctas(long long tiles) { return (int)(tiles < LOSS_PARTS ? tiles : LOSS_P
 // The three layers; GRAD: also dL/dy and the loss's partial sums for `target`.
 template <int CI, int HD, bool GRAD>
 int forward_layers(lbm_net *n, const float *x, int B, int H, int W, float *y_out,
-                   const float *target) {
+                   const float *target, const Rows &rows) {
     const __nv_bfloat16 *tb = n->theta_b;
     cudaStream_t s = n->stream;
     const Tiling g(H, W, TILE_Y);
     const long long tiles = g.tiles(B);
     if (tiles > 0x7fffffffLL) return lbm::report_error(LBM_EINVAL, "network input too large");
     const unsigned nt = TILE_QUADS * TILE_Y * (HD / 4);
-    k_conv_relu<CI, HD, true><<<(unsigned)tiles, nt, 0, s>>>(x, n->norm, n->x0, n->w_fwd,
-                                                             tb + n->off[1], g, n->a1);
-    k_conv_relu<HD, HD, false><<<(unsigned)tiles, nt, 0, s>>>(n->a1, n->norm, nullptr,
-                                                              n->w_fwd + CI * 9 * HD,
-                                                              tb + n->off[3], g, n->a2);
     const float two_n = (float)(2.0 / (double)((long long)B * H * W));
-    k_conv_out<HD, GRAD><<<out_ctas(tiles), OUT_THREADS, 0, s>>>(
-        n->a2, tb + n->off[4], tb + n->off[5], g, tiles, y_out, target, two_n, n->dy, n->loss_part);
-    NETCK(cudaGetLastError(), "network forward");
+    NETCK(lbm::launch_pdl(k_conv_relu<CI, HD, true>, (unsigned)tiles, nt, 0, s, x, n->norm, n->x0,
+                          n->w_fwd, tb + n->off[1], g, n->a1, rows),
+          "network forward");
+    NETCK(lbm::launch_pdl(k_conv_relu<HD, HD, false>, (unsigned)tiles, nt, 0, s, n->a1, n->norm,
+                          nullptr, n->w_fwd + CI * 9 * HD, tb + n->off[3], g, n->a2, Rows{}),
+          "network forward");
+    NETCK(lbm::launch_pdl(k_conv_out<HD, GRAD>, out_ctas(tiles), OUT_THREADS, 0, s, n->a2,
+                          tb + n->off[4], tb + n->off[5], g, tiles, y_out, target, two_n, n->dy,
+                          n->loss_part, rows),
+          "network forward");
     return LBM_OK;
 }
 
 template <int CI, int HD>
 int run_forward(lbm_net *n, const float *x, int B, int H, int W, float *y_out) {
-    return forward_layers<CI, HD, false>(n, x, B, H, W, y_out, nullptr);
+    return forward_layers<CI, HD, false>(n, x, B, H, W, y_out, nullptr, Rows{});
 }
 
 template <int CI, int HD>
 int run_backward(lbm_net *n, const float *x, const float *target, int B, int H, int W,
-                 const AdamArgs &adam) {
-    int st = forward_layers<CI, HD, true>(n, x, B, H, W, n->y, target);
+                 const AdamArgs &adam, const Rows &rows, int slot) {
+    int st = forward_layers<CI, HD, true>(n, x, B, H, W, n->y, target, rows);
     if (st != LBM_OK) return st;
     cudaStream_t s = n->stream;
     const Tiling g(H, W, TILE_Y), gw(H, W, WG_ROWS);
     const unsigned tiles = (unsigned)g.tiles(B), nt = TILE_QUADS * TILE_Y * (HD / 4);
-    k_conv_bwd_data<HD, 1><<<tiles, nt, 0, s>>>(n->dy, n->w_bwd + HD * 9 * HD, n->a2, g, n->dz2);
-    k_conv_bwd_data<HD, HD><<<tiles, nt, 0, s>>>(n->dz2, n->w_bwd, n->a1, g, n->dz1);
+    NETCK(lbm::launch_pdl(k_conv_bwd_data<HD, 1>, tiles, nt, 0, s, n->dy, n->w_bwd + HD * 9 * HD,
+                          n->a2, g, n->dz2),
+          "network backward");
+    NETCK(lbm::launch_pdl(k_conv_bwd_data<HD, HD>, tiles, nt, 0, s, n->dz2, n->w_bwd, n->a1, g,
+                          n->dz1),
+          "network backward");
     WgradArgs a = {n->dy, n->dz2, n->dz1, n->a2, n->a1, n->x0, {}, {}, gw.tiles(B)};
     ReduceArgs r = {};
     for (int l = 0; l < 3; ++l) {
@@ -886,16 +928,17 @@ int run_backward(lbm_net *n, const float *x, const float *target, int B, int H, 
     static_assert(smem <= 48 * 1024 && wg_smem_floats(CI, HD) <= wg_smem_floats(HD, HD) &&
                       wg_smem_floats(HD, 1) <= wg_smem_floats(HD, HD),
                   "shared memory of the weight gradients");
-    k_wgrad<CI, HD><<<a.ctas[0] + a.ctas[1] + a.ctas[2], WG_THREADS, smem, s>>>(a, gw);
+    NETCK(lbm::launch_pdl(k_wgrad<CI, HD>, a.ctas[0] + a.ctas[1] + a.ctas[2], WG_THREADS, smem, s, a, gw),
+          "network backward");
     r.loss_part = n->loss_part;
     r.loss_parts = out_ctas(g.tiles(B));
     r.n = (long long)B * H * W;
-    r.loss = n->loss_dev;
+    r.loss = n->loss_dev + slot;
     r.grad = n->grad;
     r.nparam = n->nparam;
-    k_net_reduce<<<(n->nparam + RED_PARAMS - 1) / RED_PARAMS + 1, RED_PARAMS * RED_SLICES, 0, s>>>(
-        r, adam);
-    NETCK(cudaGetLastError(), "network backward");
+    NETCK(lbm::launch_pdl(k_net_reduce, (n->nparam + RED_PARAMS - 1) / RED_PARAMS + 1,
+                          RED_PARAMS * RED_SLICES, 0, s, r, adam),
+          "network backward");
     return LBM_OK;
 }
 
@@ -946,7 +989,8 @@ LBM_API lbm_net *lbm_net_create(int cin, int hidden) {
     if (e == cudaSuccess) e = lbm::dev_alloc(&n->theta_b, sizeof(__nv_bfloat16) * o);
     if (e == cudaSuccess) e = lbm::dev_alloc(&n->loss_part, sizeof(double) * LOSS_PARTS);
     if (e == cudaSuccess)
-        e = cudaHostAlloc((void **)&n->loss_host, sizeof(double), cudaHostAllocMapped);
+        e = cudaHostAlloc((void **)&n->loss_host, sizeof(double) * (LOSS_SLOTS + 1),
+                          cudaHostAllocMapped);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&n->loss_dev, n->loss_host, 0);
     for (int l = 0; l < 3 && e == cudaSuccess; ++l)
         e = lbm::dev_alloc(&n->wpart[l],
@@ -1065,14 +1109,14 @@ LBM_API int lbm_net_forward(lbm_net *n, const float *x_dev, int batch, int h, in
 }
 
 static int backward(lbm_net *n, const float *x_dev, const float *target_dev, int batch, int h, int w,
-                    const AdamArgs &adam) {
+                    const AdamArgs &adam, const Rows &rows = Rows{}, int slot = 0) {
     if (!x_dev || !target_dev) return lbm::report_error(LBM_EINVAL, "NULL input or target");
     int st = check_shape(batch, h, w);
     if (st != LBM_OK) return st;
     st = ensure_acts(n, (long long)batch * h * w);
     if (st != LBM_OK) return st;
     NET_DISPATCH(n->cin, n->hid,
-                 (st = run_backward<CI, HD>(n, x_dev, target_dev, batch, h, w, adam)));
+                 (st = run_backward<CI, HD>(n, x_dev, target_dev, batch, h, w, adam, rows, slot)));
     if (st != LBM_OK) return st;
     n->last_pos = (long long)batch * h * w;
     return LBM_OK;
@@ -1155,6 +1199,36 @@ LBM_API int lbm_net_train_step(lbm_net *n, const float *x_dev, const float *targ
     if (!ok) return lbm_net_adam(n, lr, 0.9f, 0.999f, 1e-8f);
     n->t += 1;
     return read_loss(n, loss_host, "lbm_net_train_step");
+}
+
+LBM_API int lbm_net_train_epoch(lbm_net *n, const float *x_dev, const float *target_dev,
+                                long long nrows, const int *idx_dev, int steps, int batch, int h,
+                                int w, float lr, double *losses_host) {
+    CHECK_NET(n);
+    if (!idx_dev || steps < 0 || nrows < 1)
+        return lbm::report_error(LBM_EINVAL, "need indices, steps >= 0 and nrows >= 1");
+    // the steps are queued one behind the other; the host waits once, or where the slots are full
+    volatile int *bad = reinterpret_cast<int *>(n->loss_host + LOSS_SLOTS);
+    *bad = 0;
+    int st = LBM_OK;
+    for (int from = 0; from < steps && st == LBM_OK; from += LOSS_SLOTS) {
+        const int count = steps - from < LOSS_SLOTS ? steps - from : LOSS_SLOTS;
+        for (int k = 0; k < count && st == LBM_OK; ++k) {
+            const Rows rows = {idx_dev + (size_t)(from + k) * batch, nrows,
+                               reinterpret_cast<int *>(n->loss_dev + LOSS_SLOTS)};
+            AdamArgs a;
+            st = adam_args(n, lr, 0.9f, 0.999f, 1e-8f, &a);
+            if (st == LBM_OK) st = backward(n, x_dev, target_dev, batch, h, w, a, rows, k);
+            if (st == LBM_OK) n->t += 1;
+        }
+        NETCK(cudaStreamSynchronize(n->stream), "lbm_net_train_epoch");
+        if (st == LBM_OK && losses_host)
+            for (int k = 0; k < count; ++k)
+                losses_host[from + k] = static_cast<volatile double *>(n->loss_host)[k];
+    }
+    if (st == LBM_OK && *bad)
+        return lbm::report_error(LBM_EINVAL, "minibatch index outside the training set");
+    return st;
 }
 
 LBM_API int lbm_net_log_targets(const double *kmax_dev, long long n, float offset, float floor_k,

@@ -113,6 +113,7 @@ _SIGS = {
     "lbm_net_backward": (_i, [_vp, _vp, _vp, _i, _i, _i, _dp]),
     "lbm_net_adam": (_i, [_vp, ctypes.c_float, ctypes.c_float, ctypes.c_float, ctypes.c_float]),
     "lbm_net_train_step": (_i, [_vp, _vp, _vp, _i, _i, _i, ctypes.c_float, _dp]),
+    "lbm_net_train_epoch": (_i, [_vp, _vp, _vp, _ll, _vp, _i, _i, _i, _i, ctypes.c_float, _vp]),
     "lbm_net_log_targets": (_i, [_vp, _ll, ctypes.c_float, ctypes.c_float, _vp, _vp]),
     "lbm_net_to_maxima": (_i, [_vp, _ll, ctypes.c_float, _vp, _vp]),
     "lbm_net_log_residual": (_i, [_vp, _vp, _ll, ctypes.c_float, _vp, _vp]),
@@ -556,6 +557,13 @@ def lbm_net_adam(n, lr, beta1=0.9, beta2=0.999, eps=1e-8) -> int:
 def lbm_net_train_step(n, x_dev, t_dev, batch, h, w, lr, loss=None) -> int:
     return _ck(_lib.lbm_net_train_step(n, _ptr(x_dev), _ptr(t_dev), batch, h, w, float(lr), loss),
                "lbm_net_train_step")
+
+
+def lbm_net_train_epoch(n, x_dev, t_dev, nrows, idx_dev, steps, batch, h, w, lr, losses=None) -> int:
+    """`losses`: a contiguous float64 array of `steps` values, or None."""
+    return _ck(_lib.lbm_net_train_epoch(n, _ptr(x_dev), _ptr(t_dev), int(nrows), _ptr(idx_dev),
+                                        int(steps), int(batch), int(h), int(w), float(lr),
+                                        _ptr(losses)), "lbm_net_train_epoch")
 
 
 class Net:

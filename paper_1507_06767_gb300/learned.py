@@ -85,30 +85,19 @@ def pairs(feats, kmax):
 
 def train(net, X, T, epochs: int, batch: int, lr: float, seed: int):
     """Adam on shuffled minibatches; returns the per-epoch mean losses.  The order of the samples
-    is drawn on the host from a seeded generator; each minibatch is gathered on the device by
-    lbm_gather_rows (torch only holds the buffers)."""
+    is drawn on the host from a seeded generator; an epoch is one call, whose steps read their
+    minibatches from X and T where they lie."""
     import torch
 
     g = np.random.default_rng(np.random.SeedSequence(seed))
-    n = X.shape[0]
-    xb = torch.empty((batch,) + tuple(X.shape[1:]), dtype=X.dtype, device="cuda")
-    tb = torch.empty((batch,) + tuple(T.shape[1:]), dtype=T.dtype, device="cuda")
-    xrow, trow = X[0].numel() * X.element_size(), T[0].numel() * T.element_size()
-    bad = torch.zeros(1, dtype=torch.int32, device="cuda")
-    stream = torch.cuda.current_stream()
+    n, (h, w) = X.shape[0], X.shape[-2:]
     losses = []
     for _ in range(epochs):
         perm = torch.from_numpy(g.permutation(n).astype(np.int32)).cuda()
-        tot, cnt = 0.0, 0
-        for s in range(0, n - batch + 1, batch):
-            idx = perm[s:s + batch]
-            L.lbm_gather_rows(X, n, xrow, idx, batch, xb, bad, stream)
-            L.lbm_gather_rows(T, n, trow, idx, batch, tb, bad, stream)
-            tot += net.train_step(xb, tb, lr)
-            cnt += 1
-        losses.append(tot / max(cnt, 1))
-    if int(bad.item()):
-        raise RuntimeError("minibatch index outside the training set")
+        each = np.zeros(len(range(0, n - batch + 1, batch)))
+        if each.size:
+            L.lbm_net_train_epoch(net.n, X, T, n, perm, each.size, batch, h, w, lr, each)
+        losses.append(sum(each.tolist()) / max(each.size, 1))
     return losses
 
 

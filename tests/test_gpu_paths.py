@@ -56,3 +56,33 @@ def test_2d_runs_in_graphs_have_the_bits_of_single_steps(L, dims, periodic, dtyp
         assert np.array_equal(lats[0].sensor(8), lats[1].sensor(8))
     for lat in lats:
         lat.close()
+
+
+@pytest.mark.parametrize("cin,hidden,batch,h,w,steps", [(3, 8, 2, 12, 13, 1030),  # more than a queue
+                                                        (4, 16, 5, 33, 64, 3), (3, 16, 1, 1, 1, 2)])
+def test_an_epoch_has_the_bits_of_its_steps(L, cin, hidden, batch, h, w, steps):  # noqa: F811
+    """An epoch reads its minibatches from the training set in place and waits once; the same kernels
+    on gathered minibatches, a step at a time, give the same losses and parameters."""
+    import torch
+
+    g = seeded.rng(cin * 1000 + hidden + steps)
+    n = 3 * batch + 1
+    X = torch.from_numpy(g.normal(size=(n, cin, h, w)).astype(np.float32)).cuda()
+    T = torch.from_numpy(g.normal(size=(n, 1, h, w)).astype(np.float32)).cuda()
+    idx = torch.from_numpy(g.integers(0, n, steps * batch).astype(np.int32)).cuda()
+    nets = [L.Net(cin, hidden) for _ in range(2)]
+    theta = 0.2 * g.normal(size=nets[0].nparam)
+    for net in nets:
+        net.set_params(theta)
+    losses = np.zeros(steps)
+    L.lbm_net_train_epoch(nets[0].n, X, T, n, idx, steps, batch, h, w, 1e-3, losses)
+    for s in range(steps):
+        at = idx[s * batch:(s + 1) * batch].long()
+        assert nets[1].train_step(X[at].contiguous(), T[at].contiguous(), 1e-3) == losses[s]
+    assert np.array_equal(nets[0].params(), nets[1].params())
+    idx[-1] = n  # an index outside is not read, and refused at the end
+    with pytest.raises(L.LbmError) as ei:
+        L.lbm_net_train_epoch(nets[0].n, X, T, n, idx, steps, batch, h, w, 1e-3, None)
+    assert ei.value.status == L.LBM_EINVAL
+    for net in nets:
+        net.close()
