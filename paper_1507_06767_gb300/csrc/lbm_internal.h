@@ -84,7 +84,8 @@ cudaError_t conservation(int q, int dtype, const void *f, size_t N, double *part
 
 // Sensor reductions (lbm_aux.cu).  rtype: LBM_F64 (double maxima) or LBM_F32 (float maxima).
 cudaError_t tiles_to_blocks(int rtype, const void *tiles, int ntx, int nty, int ntz, int m, int mz,
-                            void *blocks, int nbx, int nby, int nbz, cudaStream_t s);
+                            void *blocks, int nbx, int nby, int nbz, cudaStream_t s,
+                            double *out64 = nullptr);
 cudaError_t to_f64(int rtype, const void *in, double *out, size_t n, cudaStream_t s);
 cudaError_t flags_threshold(int rtype, const void *maxima, int n, double T, int8_t *out,
                             cudaStream_t s);

@@ -189,9 +189,8 @@ extern "C" LBM_API int lbm_step_noalloc(int lattice, int dtype, int nx, int ny, 
     const int nbx = (nx + block - 1) / block, nby = (ny + block - 1) / block;
     const int nbz = (dim == 3) ? (nz + block - 1) / block : 1;
     const int rtype = (dtype == LBM_F64) ? LBM_F64 : LBM_F32;
-    e = lbm::tiles_to_blocks(rtype, tiles, ntx, nty, ntz, m, mz, blocks, nbx, nby, nbz, s);
+    e = lbm::tiles_to_blocks(rtype, tiles, ntx, nty, ntz, m, mz, blocks, nbx, nby, nbz, s,
+                             block_max_dev);
     if (e != cudaSuccess) return lbm::report_cuda_error(e, "tiles_to_blocks");
-    e = lbm::to_f64(rtype, blocks, block_max_dev, (size_t)nbx * nby * nbz, s);
-    if (e != cudaSuccess) return lbm::report_cuda_error(e, "to_f64");
     return LBM_OK;
 }
