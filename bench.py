@@ -453,9 +453,8 @@ def run_blocks(args, w, ws, rank, local):
 def run_regrid(args, w, ws, rank, local):
     """Regrid workload: the developed cavity's per-cell sensor field is tagged, buffered and
     clustered into boxes (lbm_regrid), and its block maxima mapped to levels (lbm_levels_fit); one
-    bench step is one such regrid.  lbm_regrid makes its cut decisions on the host between rounds
-    of GPU signature passes, so a regrid is timed on the host clock around the synchronising
-    call."""
+    bench step is one such regrid.  lbm_regrid returns boxes on the host, so a regrid is timed on the
+    host clock around the synchronising call."""
     import numpy as np
     import torch
 
@@ -513,14 +512,13 @@ def run_regrid(args, w, ws, rank, local):
                      "peak": peak, "unit": "GB/s",
                      "frac": round(field_bytes / (ms / 1e3) / 1e9 / peak, 4), "traffic": None,
                      "peak_kind": peak_kind,
-                     "kernel": "whole regrid (sensor-field bytes over the call's time; the call "
-                               "also waits on host decisions between signature rounds)"},
+                     "kernel": "whole regrid (sensor-field bytes over the call's time, most of "
+                               "which the clustering rounds take)"},
         "e2e": {"value": round(ms, 3), "unit": "ms", "h2d_bytes_per_step": 0,
                 "d2h_bytes_per_step": int(tags.size + 24 * len(boxes))},
-        # per step: tag pass, three 1-D dilations, one signature pass per clustering round (the
-        # rounds follow the data: 4 on this workload, profiles/launches_d3q19_256_regrid.md), and
-        # the level map's two kernels
-        "gpu_launches": args.steps * (1 + 3 + 4 + 2),
+        # per step: tag pass, three 1-D dilations, the clustering's start and the 16 rounds queued at
+        # once (those past the last box end at once), and the level map's two kernels
+        "gpu_launches": args.steps * (1 + 3 + 1 + 16 + 2),
         "clocks": clocks,
     }
     lat.close()

@@ -124,6 +124,8 @@ struct lbm_s {
     int blocks_step_form = 0;  // LBM_STEP_FORM_* for the next mesh build
     int blocks_schedule = 0;   // LBM_SCHEDULE_* for the next mesh build
 
+    lbm::rg::Work *regrid = nullptr;  // buffers of lbm_regrid
+
     // graph cache: runs of RUN_LEN[k] plain steps (k = 0: 2 steps, 1: 16 steps), by starting
     // buffer
     cudaGraphExec_t pair_exec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
@@ -505,6 +507,7 @@ LBM_API int lbm_destroy(lbm_t *h) {
     cudaFree(h->halo_msg);
     if (h->err_host) cudaFreeHost(h->err_host);
     lbm::ml::destroy(h->mesh);
+    lbm::rg::destroy(h->regrid);
     delete h;
     return LBM_OK;
 }
@@ -1311,8 +1314,8 @@ LBM_API int lbm_regrid(lbm_t *h, const double *field_dev, const lbm_regrid_param
     rp.min_width = p->min_width;
     std::vector<int> out;
     long long nt = 0;
-    int st = lbm::rg::regrid(field, ftype, h->nx, h->ny, h->nz, h->periodic, rp, p->allowed, &out,
-                             &nt, tags_out, h->stream);
+    int st = lbm::rg::regrid(&h->regrid, field, ftype, h->nx, h->ny, h->nz, h->periodic, rp,
+                             p->allowed, &out, &nt, tags_out, h->stream);
     if (st != LBM_OK) return st;
     const int n = (int)(out.size() / 6);
     *nboxes = n;

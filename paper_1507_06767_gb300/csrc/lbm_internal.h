@@ -142,7 +142,9 @@ struct Params {
     double efficiency;
     int min_width;
 };
-int regrid(const void *field, int field_type, int nx, int ny, int nz, int periodic,
+struct Work;  // a handle's buffers, made by its first regrid
+void destroy(Work *w);
+int regrid(Work **work, const void *field, int field_type, int nx, int ny, int nz, int periodic,
            const Params &p, const uint8_t *allowed_host, std::vector<int> *boxes_out,
            long long *ntagged, uint8_t *tags_out, cudaStream_t s);
 }  // namespace rg

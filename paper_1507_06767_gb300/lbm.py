@@ -904,9 +904,8 @@ class Lattice:
         tags = np.empty(tshape, dtype=np.uint8)
         boxes = (Box * max(int(max_boxes), 1))()
         n, _ = lbm_regrid(self.h, field, p, boxes, int(max_boxes), tags)
-        out = np.array([list(boxes[k].lo) + list(boxes[k].hi) for k in range(n)],
-                       dtype=np.int64).reshape(-1, 6)
-        return out, tags.astype(bool)
+        out = np.frombuffer(boxes, dtype=np.int32)[:6 * n].reshape(-1, 6).astype(np.int64)
+        return out, tags.view(bool)  # 0 or 1 each
 
     def conservation(self):
         return lbm_conservation(self.h)

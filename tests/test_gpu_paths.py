@@ -86,3 +86,39 @@ def test_an_epoch_has_the_bits_of_its_steps(L, cin, hidden, batch, h, w, steps):
     assert ei.value.status == L.LBM_EINVAL
     for net in nets:
         net.close()
+
+
+def tag_cases():
+    g = seeded.rng(4242)
+    sparse = np.zeros((1, 150, 150))
+    sparse[0, ::3, ::3] = 1.0  # 2500 boxes: more than come with the first copy, and many rounds
+    many = np.zeros((1, 300, 303))
+    many[0, ::3, ::3] = 1.0  # 10100 boxes: more than the device's queues hold
+    long = np.zeros((1, 20, 9000))  # a tag grid too long for the device's signatures
+    long[0, 3:9, g.integers(0, 9000, 30)] = 1.0
+    wide = (g.random((1, 130, 2050)) < 0.002).astype(float)
+    solid = (g.random((33, 18, 65)) < 0.03).astype(float)
+    last = np.zeros((40, 1, 1), dtype=float)
+    last[39] = 1.0
+    return {"sparse": (sparse, 1, 0), "many": (many, 1, 0), "long": (long, 1, 0),
+            "wide": (wide, 1, 1), "solid": (solid, 1, 0), "solid_w3": (solid, 3, 1), "last": (last, 1, 0)}
+
+
+@pytest.mark.parametrize("name", ["sparse", "many", "long", "wide", "solid", "solid_w3", "last"])
+def test_regrid_on_the_device_and_on_the_host(L, name):  # noqa: F811
+    """Clustering at the limits of the device's queues and beyond them, where the host takes over;
+    the buffers a handle keeps serve a second, different regrid.  Boxes and tags are whole numbers."""
+    import torch
+
+    from oracle import regrid as R
+
+    K, w, buffer = tag_cases()[name]
+    nz, ny, nx = K.shape
+    lat = L.Lattice(L.LBM_D3Q19 if nz > 1 else L.LBM_D2Q9, nx, ny, nz, 0.6, dtype=L.LBM_F64)
+    for field in (K, K[:, ::-1].copy(), K):
+        ref_boxes, ref_tags = R.regrid(field, 0.5, coarsen=1, buffer=buffer, efficiency=0.9, min_width=w)
+        boxes, tags = lat.regrid(0.5, coarsen=1, buffer=buffer, efficiency=0.9, min_width=w,
+                                 field=torch.from_numpy(field).cuda())
+        assert np.array_equal(tags, ref_tags)
+        assert boxes.tolist() == ref_boxes.tolist()
+    lat.close()
