@@ -116,7 +116,8 @@ def step_kernel_of(w, variant="auto"):
                                                  and cells >= 1 << 17)):
         return pair
     if w["dtype"] == "F64":
-        return "fused_step_f64_kernel", ("lbm_step_f64.cuh", "lbm_step.cuh", "lbm_traits.cuh")
+        # the one-cell kernel with the FP64 relaxation (fused_step_f64_kernel)
+        return "fused_step_kernel", ("lbm_step_f64.cuh", "lbm_step.cuh", "lbm_traits.cuh")
     return "fused_step_kernel", ("lbm_step.cuh", "lbm_traits.cuh")
 
 
