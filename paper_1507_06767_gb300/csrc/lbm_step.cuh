@@ -288,9 +288,19 @@ __device__ __forceinline__ typename Storage<DT>::R relax_store_cell(
     });
 }
 
+// The maxima of the warp's lanes of each tile (-1: none) into the tile's, one atomic a tile.
+__device__ __forceinline__ void combine_tile_max(int tile, int kmax, float *tile_max) {
+    const unsigned same = __match_any_sync(0xffffffffu, tile);
+    const int m = __reduce_max_sync(same, kmax);
+    if (tile >= 0 && (int)(threadIdx.x & 31) == __ffs(same) - 1)
+        atomicMax(reinterpret_cast<int *>(tile_max) + tile, m);
+}
+
 // MODE 0: no sensor.  MODE 1: sensor and per-tile max.  MODE 2: MODE 1 plus per-cell K.  HALO:
-// the faces of the slowest axis may be cuts of a slab (gather_cell).
-template <class L, int DT, int MODE, bool HALO = false>
+// the faces of the slowest axis may be cuts of a slab (gather_cell).  FLAT (no halo): a CTA takes 256
+// consecutive cells of a plane, wherever rows begin and end among them; CTAs share tiles then, whose
+// maxima they combine with atomics in a buffer that the sensor step before has cleared.
+template <class L, int DT, int MODE, bool HALO = false, bool FLAT = false>
 __global__ void __launch_bounds__(CTA_X *CTA_Y, LBM_STEP_MIN_BLOCKS)
     fused_step_kernel(const typename Storage<DT>::T *__restrict__ fin,
                       typename Storage<DT>::T *__restrict__ fout, const StepParams p,
@@ -302,11 +312,13 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, LBM_STEP_MIN_BLOCKS)
     constexpr int Q = L::Q;
     constexpr int ZT = (L::D == 3) ? TILE : 1;
 
-    const int lane = threadIdx.x;
-    const int x = blockIdx.x * CTA_X + lane;
-    const int y = blockIdx.y * CTA_Y + threadIdx.y;
-    const int z0 = blockIdx.z * ZT;
+    static_assert(!FLAT || !HALO, "flat rows have no halo");
     const int nx = p.nx, ny = p.ny, nz = p.nz;
+    const int lane = threadIdx.x;
+    const int at = blockIdx.x * (CTA_X * CTA_Y) + threadIdx.y * CTA_X + lane;  // FLAT: in the plane
+    const int y = FLAT ? at / nx : blockIdx.y * CTA_Y + threadIdx.y;
+    const int x = FLAT ? at - y * nx : blockIdx.x * CTA_X + lane;
+    const int z0 = blockIdx.z * ZT;
     const bool active = (x < nx) && (y < ny);
     const size_t N = (size_t)nx * ny * nz;
     const R omega = param_omega<R>(p);
@@ -326,9 +338,13 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, LBM_STEP_MIN_BLOCKS)
 
     B kmax = 0;
     // a warp is one row of 32 cells: when the row and all its pull sources lie inside the lattice
-    // (a warp-uniform test) the gather needs no wall or wrap logic
-    const bool inner_x = blockIdx.x * CTA_X >= 1 && (blockIdx.x + 1) * CTA_X <= nx - 1;
-    const bool inner_y = y >= 1 && y <= ny - 2;
+    // (a warp-uniform test) the gather needs no wall or wrap logic.  FLAT: 32 cells of one row or more.
+    bool inner_x = blockIdx.x * CTA_X >= 1 && (blockIdx.x + 1) * CTA_X <= nx - 1;
+    bool inner_y = y >= 1 && y <= ny - 2;
+    if constexpr (FLAT) {
+        inner_x = __all_sync(0xffffffffu, !active || (x >= 1 && x <= nx - 2));
+        inner_y = __all_sync(0xffffffffu, !active || inner_y);
+    }
 
     for (int dz = 0; dz < ZT; ++dz) {
         const int z = z0 + dz;
@@ -352,7 +368,10 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, LBM_STEP_MIN_BLOCKS)
         }
     }
 
-    if (MODE != 0) {
+    if constexpr (FLAT && MODE != 0)
+        combine_tile_max(active ? (blockIdx.z * p.nty + y / TILE) * p.ntx + x / TILE : -1, kmax,
+                         tile_max);
+    if (!FLAT && MODE != 0) {
         // max over the 8 lanes of each x-tile of this row, then over the 8 rows via shared memory
 #pragma unroll
         for (int off = 4; off >= 1; off >>= 1) {
@@ -386,6 +405,31 @@ inline cudaError_t launch_step_kernel(void (*kernel)(Params...), dim3 grid, dim3
     return cudaGetLastError();
 }
 
+// Whether a step takes the cells of a plane in a line (FLAT) rather than in rows of CTA_X lanes; dtype
+// and the cells a lane takes along x as in the kernels.  Rows that do not fill whole warps leave lanes
+// idle and start anywhere in a memory sector, a line neither (rows -> line, us a plain step: 195 x 129 x
+// 97 FP32 76.3 -> 64.7, FP64 886 -> 773; 250 x 182 x 130 FP32 174 -> 144, BF16 101 -> 95; 100^3 FP16
+// 29.7 -> 22.4; sensor steps of 100^3 FP32 39.2 -> 35.0).  Two cells a lane gain in long rows too, as a
+// CTA then reads longer runs (256 x 256 x 128 FP16 124 -> 120, 128 x 128 x 64 unchanged); one cell a lane
+// does not (256 x 256 x 64 FP32 101.0 -> 100.4), and two lose in sensor steps (250 x 182 x 130 BF16 102
+// -> 105).  Below 2^19 cells the line has fewer than two CTAs an SM, where rows have more and smaller ones
+// (42 x 36 x 227 FP32 18.7 -> 19.8 a sensor step, 40^3 9.8 -> 10.1), except in FP64, which the FP64 units
+// bound (40^3 41 -> 29).  In 2-D
+// FP64 (130^2 6.3 -> 4.9) and FP32 (50 x 700 2.10 -> 1.84, 301 x 203 2.22 -> 2.09) gain, 16-bit types
+// lose (1025 x 1023 10.0 -> 10.5).
+template <class L>
+inline bool flat_rows(const StepParams &p, int mode, int dtype, int per_lane) {
+    const long long plane = (long long)p.nx * p.ny;
+    if (plane >= 1LL << 30) return false;  // the kernels count a plane's cells in ints
+    const bool ragged = p.nx % (CTA_X * per_lane) != 0;
+    if (dtype == 0) return mode == 0 && ragged;
+    if (L::D == 2) return mode == 0 && ragged && dtype == 1 && per_lane == 1;
+    if (plane * p.nz < 1LL << 19) return false;
+    // a sensor step's tile maxima are combined in a buffer that has to be clear
+    if (mode != 0) return ragged && per_lane == 1 && p.tile_zero;
+    return ragged || (per_lane == 2 && p.nx >= 256);
+}
+
 template <class L, int DT, bool HALO = false>
 cudaError_t launch_fused_step(const void *fin, void *fout, const StepParams &p, int mode,
                               void *tile_max, void *k_field, cudaStream_t stream) {
@@ -398,6 +442,16 @@ cudaError_t launch_fused_step(const void *fin, void *fout, const StepParams &p, 
     T *b = static_cast<T *>(fout);
     R *tm = static_cast<R *>(tile_max);
     R *kf = static_cast<R *>(k_field);
+    if constexpr (!HALO && DT != 0) {
+        if (flat_rows<L>(p, mode, DT, 1)) {
+            grid.x = (unsigned)(((long long)p.nx * p.ny + CTA_X * CTA_Y - 1) / (CTA_X * CTA_Y));
+            grid.y = 1;
+            return launch_step_kernel<L>(mode == 0   ? fused_step_kernel<L, DT, 0, false, true>
+                                         : mode == 1 ? fused_step_kernel<L, DT, 1, false, true>
+                                                     : fused_step_kernel<L, DT, 2, false, true>,
+                                         grid, block, 0, stream, a, b, p, tm, kf);
+        }
+    }
     if (mode == 0)
         return launch_step_kernel<L>(fused_step_kernel<L, DT, 0, HALO>, grid, block, 0, stream, a, b, p, tm, kf);
     if (mode == 1)

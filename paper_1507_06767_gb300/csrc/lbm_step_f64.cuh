@@ -127,12 +127,12 @@ __device__ __forceinline__ double relax_cell_f64(const double *df, const RelaxF6
 
 constexpr int F64_SPREAD_CTAS = 512;  // CTAs wanted of a plain step on a small 2-D lattice (152 SMs)
 
-// MODE and HALO as in fused_step_kernel.  A CTA covers whole tiles as there where the step records
+// MODE, HALO and FLAT as in fused_step_kernel.  A CTA covers whole tiles as there where the step records
 // the tile maxima; a plain step takes one plane a CTA in 3-D and, on small 2-D lattices, fewer rows
 // (blockDim.y), as it is bound by the FP64 units: short CTAs shorten the last wave (128^3: 0.716 ms a
 // step against 0.724 with two planes and 0.737 with four) and reach every SM (128^2: 512 CTAs of one
 // row, 64 of eight).  The planes' CTAs come in a line, as there may be more than a grid's z takes.
-template <class L, int MODE, bool HALO>
+template <class L, int MODE, bool HALO, bool FLAT = false>
 __global__ void __launch_bounds__(CTA_X *CTA_Y, 2)
     fused_step_f64_kernel(const double *__restrict__ fin, double *__restrict__ fout,
                           const StepParams p, double *__restrict__ tile_max,
@@ -140,10 +140,14 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, 2)
     constexpr int Q = L::Q;
     constexpr int ZT = MODE != 0 && L::D == 3 ? TILE : 1;
     const int nx = p.nx, ny = p.ny, nz = p.nz;
-    const int gx = (nx + CTA_X - 1) / CTA_X, gy = (ny + blockDim.y - 1) / blockDim.y;
+    const int cta = CTA_X * blockDim.y;
+    const int gx = FLAT ? (nx * ny + cta - 1) / cta : (nx + CTA_X - 1) / CTA_X;
+    const int gy = FLAT ? 1 : (ny + blockDim.y - 1) / blockDim.y;
     const int bx = blockIdx.x % gx, by = blockIdx.x / gx % gy, bz = blockIdx.x / gx / gy;
     const int lane = threadIdx.x;
-    const int x = bx * CTA_X + lane, y = by * blockDim.y + threadIdx.y, z0 = bz * ZT;
+    const int at = bx * cta + threadIdx.y * CTA_X + lane;  // FLAT: in the plane
+    const int y = FLAT ? at / nx : by * blockDim.y + threadIdx.y;
+    const int x = FLAT ? at - y * nx : bx * CTA_X + lane, z0 = bz * ZT;
     const bool active = (x < nx) && (y < ny);
     const size_t N = (size_t)nx * ny * nz;
     if constexpr (L::D == 2) fin = pdl_wait(fin);
@@ -154,8 +158,12 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, 2)
             static_cast<double *>(p.tile_zero)[t] = 0.0;
     }
     long long kmax = 0;
-    const bool inner_x = bx * CTA_X >= 1 && (bx + 1) * CTA_X <= nx - 1;
-    const bool inner_y = y >= 1 && y <= ny - 2;
+    bool inner_x = bx * CTA_X >= 1 && (bx + 1) * CTA_X <= nx - 1;
+    bool inner_y = y >= 1 && y <= ny - 2;
+    if constexpr (FLAT) {
+        inner_x = __all_sync(0xffffffffu, !active || (x >= 1 && x <= nx - 2));
+        inner_y = __all_sync(0xffffffffu, !active || inner_y);
+    }
     for (int dz = 0; dz < ZT; ++dz) {
         const int z = z0 + dz;
         if (z >= nz) break;
@@ -207,11 +215,19 @@ cudaError_t launch_fused_step_f64(const void *fin, void *fout, const StepParams 
     int rows = CTA_Y;
     if (L::D == 2 && mode == 0)
         while (rows > 1 && gx * ((p.ny + rows - 1) / rows) < F64_SPREAD_CTAS) rows /= 2;
-    const dim3 block(CTA_X, rows), grid((unsigned)(gx * ((p.ny + rows - 1) / rows) * gz));
+    const dim3 block(CTA_X, rows);
+    dim3 grid((unsigned)(gx * ((p.ny + rows - 1) / rows) * gz));
     const double *a = static_cast<const double *>(fin);
     double *b = static_cast<double *>(fout), *tm = static_cast<double *>(tile_max),
            *kf = static_cast<double *>(k_field);
     const RelaxF64 k(p);
+    if constexpr (!HALO) {
+        if (mode == 0 && flat_rows<L>(p, mode, 0, 1)) {
+            grid.x = (unsigned)(((long long)p.nx * p.ny + CTA_X * rows - 1) / (CTA_X * rows) * gz);
+            return launch_step_kernel<L>(fused_step_f64_kernel<L, 0, false, true>, grid, block, 0,
+                                         stream, a, b, p, tm, kf, k);
+        }
+    }
     if (mode == 0)
         return launch_step_kernel<L>(fused_step_f64_kernel<L, 0, HALO>, grid, block, 0, stream, a, b, p, tm, kf, k);
     if (mode == 1)

@@ -190,7 +190,34 @@ __device__ __forceinline__ float2 relax_pair(Get1 &&moments, Get2 &&relax, float
     return __fmul2_rn(ksum, f2(1.f / (float)Q));
 }
 
-template <class L, int DT, int MODE>
+// The order in which FLAT steps take the pairs of cells of a plane: the rows between the y
+// faces one after the other, contiguous in memory, then the two rows on the faces, each starting a
+// warp, so that a warp's cells are all inside in y or all on a face.  No lane is left over at the end
+// of a row but the faces'.
+struct FlatLine {
+    int width, ny;            // units of a row
+    int inner, inner_r, row;  // units inside in y; the same and a row in whole warps
+    __host__ __device__ FlatLine(int w, int n)
+        : width(w), ny(n), inner(n > 2 ? (n - 2) * w : 0), inner_r((inner + 31) & ~31), row((w + 31) & ~31) {}
+    __host__ __device__ unsigned ctas(int threads) const {
+        return (unsigned)((inner_r + 2LL * row + threads - 1) / threads);
+    }
+    // unit x of row y of place `at`; x = width where there is none
+    __device__ __forceinline__ void cell(int at, int &x, int &y) const {
+        if (at < inner_r) {
+            y = 1 + at / width;
+            x = at < inner ? at - (y - 1) * width : width;
+            return;
+        }
+        at -= inner_r;
+        y = at < row ? 0 : ny - 1;
+        x = at < row ? at : at - row;
+        if (x > width || (at >= row && ny == 1)) x = width;
+    }
+};
+
+// FLAT (MODE 0): the pairs of a plane in the order of FlatLine rather than in rows of 32 lanes.
+template <class L, int DT, int MODE, bool FLAT = false>
 __global__ void __launch_bounds__(CTA_X *CTA_Y, DT == 1 ? LBM_PAIR_MIN_BLOCKS_F32 : LBM_PAIR_MIN_BLOCKS)
     fused_step_pair_kernel(const typename Storage<DT>::T *__restrict__ fin,
                            typename Storage<DT>::T *__restrict__ fout, const StepParams p,
@@ -202,11 +229,14 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, DT == 1 ? LBM_PAIR_MIN_BLOCKS_F3
     constexpr int Q = L::Q;
     constexpr int ZT = (L::D == 3) ? TILE : 1;
 
-    const int lane = threadIdx.x;
-    const int x0 = (blockIdx.x * CTA_X + lane) * 2;
-    const int y = blockIdx.y * CTA_Y + threadIdx.y;
-    const int z0 = blockIdx.z * ZT;
+    static_assert(!FLAT || MODE == 0, "tiles need rows");
     const int nx = p.nx, ny = p.ny, nz = p.nz;
+    const int lane = threadIdx.x;
+    int pair = blockIdx.x * CTA_X + lane, y = blockIdx.y * CTA_Y + threadIdx.y;
+    if constexpr (FLAT)
+        FlatLine(nx / 2, ny).cell(blockIdx.x * (CTA_X * CTA_Y) + threadIdx.y * CTA_X + lane, pair, y);
+    const int x0 = pair * 2;
+    const int z0 = blockIdx.z * ZT;
     const bool active = (x0 < nx) && (y < ny);
     // element offsets fit in 32 bits: (q + 1) * cells < 2^32
     const unsigned N = (unsigned)nx * (unsigned)ny * (unsigned)nz;
@@ -227,7 +257,7 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, DT == 1 ? LBM_PAIR_MIN_BLOCKS_F3
     for (int dz = 0; dz < ZT; ++dz) {
         const int z = z0 + dz;
         if (z >= nz) break;
-        // y and z are warp-uniform (a warp is one row); x0 is not
+        // z is warp-uniform, and so is whether y is inside (FlatLine; else a warp is one row); x0 is not
         const bool inner_yz = (y > 0) && (y < ny - 1) && (L::D == 2 || ((z > 0) && (z < nz - 1)));
         const bool interior = inner_yz && (x0 > 0) && (x0 + 2 < nx);
         const bool fast = __all_sync(0xffffffffu, !active || interior);
@@ -348,6 +378,12 @@ cudaError_t launch_fused_step_pair(const void *fin, void *fout, const StepParams
     T *b = static_cast<T *>(fout);
     float *tm = static_cast<float *>(tile_max);
     float *kf = static_cast<float *>(k_field);
+    if (flat_rows<L>(p, mode, DT, 2)) {
+        grid.x = FlatLine(p.nx / 2, p.ny).ctas(CTA_X * CTA_Y);
+        grid.y = 1;
+        return launch_step_kernel<L>(fused_step_pair_kernel<L, DT, 0, true>, grid, block, 0, stream, a,
+                                     b, p, tm, kf);
+    }
     if (mode == 0)
         return launch_step_kernel<L>(fused_step_pair_kernel<L, DT, 0>, grid, block, 0, stream, a, b, p, tm, kf);
     if (mode == 1)

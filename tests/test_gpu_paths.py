@@ -122,3 +122,51 @@ def test_regrid_on_the_device_and_on_the_host(L, name):  # noqa: F811
         assert np.array_equal(tags, ref_tags)
         assert boxes.tolist() == ref_boxes.tolist()
     lat.close()
+
+
+@pytest.mark.parametrize("dtype", ["LBM_F32", "LBM_F16S", "LBM_BF16S"])
+@pytest.mark.parametrize("dims,periodic", [((1, 725, 724), 0), ((33, 180, 90), 5), ((99, 80, 80), 0),
+                                           ((257, 3, 681), 3), ((5000, 2, 53), 4), ((33, 180, 80), 7)])
+def test_3d_steps_in_a_line_have_the_bits_of_rows(L, dims, periodic, dtype):  # noqa: F811
+    """Sensor steps that take a plane's cells in a line, whose CTAs share tiles (from 2^19 cells on, the
+    last case below), against the allocation-free call, which keeps to rows: populations and maxima, with
+    the tile buffers alternating."""
+    import torch
+
+    nx, ny, nz = dims
+    o = O.Oracle(19, *dims, tau=0.7, lid=(0.1, 0.0, 0.02), periodic=periodic)
+    lat = L.Lattice(19, *dims, 0.7, dtype=getattr(L, dtype), lid=(0.1, 0.02), periodic=periodic)
+    lat.set_populations(perturbed(o, seed=7 + sum(dims), amp=0.02))
+    L.lbm_set_sensor_every(lat.h, 1)
+    src = torch.from_numpy(lat.raw().copy()).cuda()
+    dst = torch.empty_like(src)
+    maxima = torch.empty(L.lbm_nblocks(lat.h, 8), dtype=torch.float64, device="cuda")
+    for _ in range(4):
+        lat.step(1)
+        L.lbm_step_noalloc(19, getattr(L, dtype), nx, ny, nz, 0.7, 0.1, 0.02, periodic, src, dst, 8, maxima,
+                           torch.cuda.current_stream())
+        torch.cuda.synchronize()
+        assert np.array_equal(lat.raw(), dst.cpu().numpy())
+        assert np.array_equal(lat.sensor(8), maxima.cpu().numpy())
+        src, dst = dst, src
+    lat.close()
+
+
+@pytest.mark.parametrize("dtype", ["LBM_F64", "LBM_F32", "LBM_F16S", "LBM_BF16S"])
+@pytest.mark.parametrize("q,dims,periodic", [(19, (99, 80, 80), 0), (19, (98, 80, 80), 5), (19, (2, 600, 440), 0),
+                                             (19, (256, 3, 683), 2), (19, (9, 7, 33), 7), (9, (45, 61, 1), 0),
+                                             (9, (33, 1, 1), 0), (9, (700, 3, 1), 3)])
+def test_plain_steps_in_a_line_match_the_oracle(L, q, dims, periodic, dtype):  # noqa: F811
+    """Plain steps over a plane's cells in a line, one and two cells a lane, at sides where rows, faces
+    and the last warp end anywhere.  Two steps round a population a few times at the type's precision
+    relative to the largest one (16-bit types: that of f - w, here under 0.1 of it)."""
+    o = O.Oracle(q, *dims, tau=0.8, lid=(0.1, 0.0, 0.0), periodic=periodic)
+    lat = L.Lattice(q, *dims, 0.8, dtype=getattr(L, dtype), lid=(0.1, 0.0), periodic=periodic)
+    lat.set_populations(perturbed(o, seed=3 + sum(dims), amp=0.02))
+    f = lat.populations()  # as stored
+    L.lbm_set_sensor_every(lat.h, 1000)
+    lat.step(2)
+    for _ in range(2):
+        f, _, _, _ = o.step(f, sensor=False)
+    assert rel(lat.populations(), f) <= {"LBM_F64": 1e-14, "LBM_F32": 2e-6, "LBM_F16S": 2e-4, "LBM_BF16S": 2e-3}[dtype]
+    lat.close()
