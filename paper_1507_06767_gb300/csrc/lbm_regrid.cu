@@ -289,7 +289,8 @@ struct ClusterState {
     int count[CL_ROUNDS + 1];  // boxes of each round
     int used[CL_ROUNDS + 1];   // signature words of each round
     int accepted;
-    int overflow;              // a queue or pool was too small: the host clusters instead
+    int overflow;              // a queue or pool was too small: the host, which alone reads this,
+                               // clusters instead
     long long tagged;
     HBox boxes[CL_BOXES];      // the accepted ones
 };
@@ -359,12 +360,13 @@ __device__ int decide_warp(HBox &box, const int *s, double efficiency, int wmin,
             }
         }
         first[a] = __reduce_min_sync(0xffffffffu, lo);
-        len[a] = __reduce_max_sync(0xffffffffu, hi) - first[a] + 1;
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        if (hi < 0) return 0;  // no tag on this axis, so none in the box
+        len[a] = hi - first[a] + 1;
         sig[a] = at + first[a];
         at += n;
     }
     for (int off = 16; off >= 1; off >>= 1) total += __shfl_xor_sync(0xffffffffu, total, off);
-    if (total == 0) return 0;
     for (int a = 0; a < 3; ++a) {
         box.lo[a] += first[a];
         box.hi[a] = box.lo[a] + len[a];
@@ -413,8 +415,11 @@ __global__ void __launch_bounds__(CL_THREADS)
     __shared__ int sx[CL_EXTENTS];
     __shared__ int last;
     ClusterState &st = w->state;
+    // The round's boxes and signature words are what the launches before left, the same for every
+    // thread of this one: all go on or all leave, whatever other CTAs of the launch queue meanwhile.
+    // Counts beyond the limits are of boxes that have no place: the clustering has failed.
     const int count = st.count[round];
-    if (count == 0 || st.overflow) return;
+    if (count == 0 || count > CL_BOXES || st.used[round] > CL_SIG) return;
     const int parts = min(max((int)gridDim.x / count, 1), CL_MAX_PARTS);
     DBox *queue = w->queue[round & 1];
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;

@@ -170,3 +170,34 @@ def test_plain_steps_in_a_line_match_the_oracle(L, q, dims, periodic, dtype):  #
         f, _, _, _ = o.step(f, sensor=False)
     assert rel(lat.populations(), f) <= {"LBM_F64": 1e-14, "LBM_F32": 2e-6, "LBM_F16S": 2e-4, "LBM_BF16S": 2e-3}[dtype]
     lat.close()
+
+
+@pytest.mark.parametrize("name", ["boxes_w2", "rows"])
+def test_regrid_beyond_the_queues_while_other_work_runs(L, name):  # noqa: F811
+    """Rounds that outgrow the device's queues: more than 8192 boxes of width 2 in a round, and rows whose signatures
+    outgrow the pool.  Steps of another lattice hold the SMs, so that CTAs of one launch start at
+    different times, before and after one of them finds a queue full; the boxes are the host's."""
+    import torch
+
+    from oracle import regrid as R
+
+    if name == "rows":
+        K, w = np.zeros((1, 1500, 1500)), 1
+        K[0, ::3] = 1.0
+    else:
+        K, w = np.zeros((1, 650, 655)), 2
+        K[0, ::5, ::5] = K[0, 1::5, ::5] = K[0, ::5, 1::5] = K[0, 1::5, 1::5] = 1.0
+    ref_boxes, ref_tags = R.regrid(K, 0.5, coarsen=1, buffer=0, efficiency=0.9, min_width=w)
+    assert name == "rows" or len(ref_boxes) > 8192
+    lat = L.Lattice(L.LBM_D2Q9, K.shape[2], K.shape[1], 1, 0.6, dtype=L.LBM_F64)
+    field = torch.from_numpy(K).cuda()
+    side = torch.cuda.Stream()
+    other = L.Lattice(L.LBM_D3Q19, 128, 128, 128, 0.6, dtype=L.LBM_F32, stream=side)
+    for _ in range(3):
+        other.step(200)
+        boxes, tags = lat.regrid(0.5, coarsen=1, buffer=0, efficiency=0.9, min_width=w, field=field)
+        assert np.array_equal(tags, ref_tags)
+        assert boxes.tolist() == ref_boxes.tolist()
+    side.synchronize()
+    other.close()
+    lat.close()
