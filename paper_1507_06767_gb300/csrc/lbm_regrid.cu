@@ -544,11 +544,13 @@ int cluster(Work &wk, const uint8_t *tags, int tx, int ty, int tz, const Params 
     if (fresh || !wk.sig_clear) RGCK(cudaMemsetAsync(w->sig, 0, sizeof(w->sig), s), "memset(signatures)");
     wk.sig_clear = false;
     const ClusterState *head = static_cast<const ClusterState *>(wk.head);
+    // a piece wider than any extent is as inadmissible as one of INT_MAX, to which lanes cannot be added
+    const int wmin = std::min(p.min_width, CL_EXTENTS + 1);
     for (bool first = true;; first = false) {
         k_cluster_start<<<1, 1, 0, s>>>(w, tx, ty, tz, first);
         for (int r = 0; r < CL_ROUNDS; ++r)
             k_cluster_round<<<CL_CTAS, CL_THREADS, 0, s>>>(tags, tx, ty, w, r, first && r == 0,
-                                                          p.efficiency, p.min_width);
+                                                          p.efficiency, wmin);
         RGCK(cudaGetLastError(), "clustering kernel");
         RGCK(cudaMemcpyAsync(wk.head, w, CL_HEAD, cudaMemcpyDeviceToHost, s), "boxes");
         if (first && tags_out)

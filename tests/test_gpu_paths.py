@@ -201,3 +201,21 @@ def test_regrid_beyond_the_queues_while_other_work_runs(L, name):  # noqa: F811
     side.synchronize()
     other.close()
     lat.close()
+
+
+@pytest.mark.parametrize("w", [9, 66, 8193, 2 ** 31 - 31, 2 ** 31 - 1])
+def test_regrid_with_pieces_wider_than_the_grid(L, w):  # noqa: F811
+    """A least width that few or no cuts leave, up to the largest int: one box, or the oracle's few."""
+    import torch
+
+    from oracle import regrid as R
+
+    K = (seeded.rng(99).random((33, 18, 65)) < 0.03).astype(float)
+    lat = L.Lattice(L.LBM_D3Q19, 65, 18, 33, 0.6, dtype=L.LBM_F64)
+    ref_boxes, ref_tags = R.regrid(K, 0.5, coarsen=1, buffer=0, efficiency=0.9, min_width=w)
+    assert (len(ref_boxes) == 1) == (w > 9)
+    boxes, tags = lat.regrid(0.5, coarsen=1, buffer=0, efficiency=0.9, min_width=w,
+                             field=torch.from_numpy(K).cuda())
+    assert np.array_equal(tags, ref_tags)
+    assert boxes.tolist() == ref_boxes.tolist()
+    lat.close()
