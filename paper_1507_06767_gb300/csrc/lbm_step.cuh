@@ -288,6 +288,12 @@ __device__ __forceinline__ typename Storage<DT>::R relax_store_cell(
     });
 }
 
+// The halo planes are read behind pdl_wait too: the launch before the step may have filled them.
+__device__ __forceinline__ void order_halos(StepParams &p) {
+    p.halo_lo = pdl_order(p.halo_lo);
+    p.halo_hi = pdl_order(p.halo_hi);
+}
+
 // The maxima of the warp's lanes of each tile (-1: none) into the tile's, one atomic a tile.
 __device__ __forceinline__ void combine_tile_max(int tile, int kmax, float *tile_max) {
     const unsigned same = __match_any_sync(0xffffffffu, tile);
@@ -303,7 +309,7 @@ __device__ __forceinline__ void combine_tile_max(int tile, int kmax, float *tile
 template <class L, int DT, int MODE, bool HALO = false, bool FLAT = false>
 __global__ void __launch_bounds__(CTA_X *CTA_Y, LBM_STEP_MIN_BLOCKS)
     fused_step_kernel(const typename Storage<DT>::T *__restrict__ fin,
-                      typename Storage<DT>::T *__restrict__ fout, const StepParams p,
+                      typename Storage<DT>::T *__restrict__ fout, StepParams p,
                       typename Storage<DT>::R *__restrict__ tile_max,
                       typename Storage<DT>::R *__restrict__ k_field) {
     using S = Storage<DT>;
@@ -324,6 +330,7 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, LBM_STEP_MIN_BLOCKS)
     const R omega = param_omega<R>(p);
 
     if constexpr (L::D == 2) fin = pdl_wait(fin);
+    if constexpr (L::D == 2 && HALO) order_halos(p);
 
     // clear the other tile buffer for the next sensor step (kernels that combine tiles across
     // CTAs with atomics need it zeroed)

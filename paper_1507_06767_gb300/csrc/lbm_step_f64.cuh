@@ -135,7 +135,7 @@ constexpr int F64_SPREAD_CTAS = 512;  // CTAs wanted of a plain step on a small 
 template <class L, int MODE, bool HALO, bool FLAT = false>
 __global__ void __launch_bounds__(CTA_X *CTA_Y, 2)
     fused_step_f64_kernel(const double *__restrict__ fin, double *__restrict__ fout,
-                          const StepParams p, double *__restrict__ tile_max,
+                          StepParams p, double *__restrict__ tile_max,
                           double *__restrict__ k_field, const RelaxF64 k) {
     constexpr int Q = L::Q;
     constexpr int ZT = MODE != 0 && L::D == 3 ? TILE : 1;
@@ -151,6 +151,7 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, 2)
     const bool active = (x < nx) && (y < ny);
     const size_t N = (size_t)nx * ny * nz;
     if constexpr (L::D == 2) fin = pdl_wait(fin);
+    if constexpr (L::D == 2 && HALO) order_halos(p);
     if (MODE != 0 && p.tile_zero) {  // as in fused_step_kernel
         const size_t nt = (size_t)p.ntx * p.nty * p.ntz, me = (size_t)blockIdx.x * (CTA_X * CTA_Y) +
                                                               threadIdx.y * CTA_X + lane;

@@ -219,3 +219,33 @@ def test_regrid_with_pieces_wider_than_the_grid(L, w):  # noqa: F811
     assert np.array_equal(tags, ref_tags)
     assert boxes.tolist() == ref_boxes.tolist()
     lat.close()
+
+
+@pytest.mark.parametrize("dtype", ["LBM_F64", "LBM_F32", "LBM_F16S", "LBM_BF16S"])
+@pytest.mark.parametrize("nx,ny", [(33, 17), (700, 303)])
+def test_2d_slab_steps_read_the_halos_just_filled(L, nx, ny, dtype):  # noqa: F811
+    """A 2-D slab that is its own neighbour, its halos filled from the device by the launch before each
+    step and nothing waited for: the bits of a lattice that is periodic along the cut axis."""
+    import torch
+
+    o = O.Oracle(9, nx, ny, 1, tau=0.7, lid=(0.0, 0.0, 0.0), periodic=2)
+    f = perturbed(o, seed=11 + nx, amp=0.02)
+    whole, slab = [L.Lattice(9, nx, ny, 1, 0.7, dtype=getattr(L, dtype), lid=(0.0, 0.0), periodic=p)
+                   for p in (2, 0)]
+    slab.set_halo(L.LBM_HALO_LO | L.LBM_HALO_HI)
+    for lat in (whole, slab):
+        L.lbm_set_kernel_variant(lat.h, L.LBM_KERNEL_CELL)
+        L.lbm_set_sensor_every(lat.h, 7)
+        lat.set_populations(f)
+    up, down = [torch.empty(L.lbm_halo_size(slab.h)[1], dtype=torch.uint8, device="cuda") for _ in range(2)]
+    for _ in range(50):
+        L.lbm_halo_export(slab.h, L.LBM_HALO_HI, up)
+        L.lbm_halo_export(slab.h, L.LBM_HALO_LO, down)
+        L.lbm_halo_import(slab.h, L.LBM_HALO_LO, up)
+        L.lbm_halo_import(slab.h, L.LBM_HALO_HI, down)
+        slab.step(1)
+        whole.step(1)
+    assert np.array_equal(slab.raw(), whole.raw())
+    assert np.array_equal(slab.sensor(8), whole.sensor(8))
+    for lat in (whole, slab):
+        lat.close()
