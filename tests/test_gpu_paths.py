@@ -249,3 +249,26 @@ def test_2d_slab_steps_read_the_halos_just_filled(L, nx, ny, dtype):  # noqa: F8
     assert np.array_equal(slab.sensor(8), whole.sensor(8))
     for lat in (whole, slab):
         lat.close()
+
+
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("q,dims,c5", [(9, (40, 33, 1), (1, 1, 0)), (19, (20, 17, 24), (0, 0, 1))])
+def test_fp64_nan_maxima_stand_out(L, q, dims, c5, value):  # noqa: F811
+    """One infinite or NaN population makes K NaN, of either sign, in the cell it arrives at: its block's
+    maximum is NaN and flagged, the others are those of a run without it."""
+    o = O.Oracle(q, *dims, tau=0.7, lid=(0.0, 0.0, 0.0))
+    f = perturbed(o, seed=41, amp=0.02)
+    lat = L.Lattice(q, *dims, 0.7, dtype=L.LBM_F64, lid=(0.0, 0.0))
+    maxima = []
+    x, y, z = (n // 2 for n in dims)
+    for v in (f[5, z, y, x], value):
+        f[5, z, y, x] = v
+        lat.set_populations(f)
+        lat.step(1)
+        maxima.append(lat.sensor(8).reshape([-(-n // 8) for n in dims[::-1]]))
+    hit = np.zeros_like(maxima[0], dtype=bool)
+    hit[(z + c5[2]) // 8, (y + c5[1]) // 8, (x + c5[0]) // 8] = True
+    assert np.array_equal(np.isnan(maxima[1]), hit)
+    assert np.array_equal(maxima[1][~hit], maxima[0][~hit])
+    assert lat.flag(1e300, block=8).reshape(hit.shape)[hit] > 0
+    lat.close()
