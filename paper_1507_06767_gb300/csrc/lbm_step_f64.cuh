@@ -35,6 +35,14 @@ __device__ __forceinline__ Fraction operator+(const Fraction &a, const Fraction 
     return {fma(a.num, b.den, b.num * a.den), a.den * b.den};
 }
 
+// Whether |v| lies within 2^-300 .. 2^300, and whether v is finite, from the exponent.
+__device__ __forceinline__ bool mid_range(double v) {
+    return ((unsigned)__double2hiint(v) >> 20 & 0x7ff) - (1023 - 300) <= 600;
+}
+__device__ __forceinline__ bool is_finite(double v) {
+    return ((unsigned)__double2hiint(v) >> 20 & 0x7ff) != 0x7ff;
+}
+
 // Moments, equilibrium, sensor and BGK collision of one cell from its gathered deviations df, as
 // relax_cell; emit(i, d) receives the post-collision deviation of every population.
 //
@@ -45,8 +53,9 @@ __device__ __forceinline__ Fraction operator+(const Fraction &a, const Fraction 
 //     M = (1 - omega) / 2 m + 3 omega w c.j,   B = rho - 1 - 1.5 j.j / rho,
 // where j = rho u.  The momentum is scaled once by 3 omega w (w the diagonal weight), so that c.j is
 // one addition in both S and M.  The sensor's fractions |f^neq| / f^eq are added over common
-// denominators, three opposite pairs (two in 2-D) to one division; a few pairs only, so that the
-// product of equilibria stays in range for densities from 1e-40 to 1e40.
+// denominators, three opposite pairs (two in 2-D) to one division.  Where a pair's product of equilibria
+// is far from one (densities beyond 1e45, zeros, infinities, NaN) or the numerator overflows, that
+// group's fractions are divided one by one, as the products of three pairs would leave the range.
 //
 // A plain D3Q19 step issues about 165 FP64 instructions a cell (about 350 with each direction relaxed
 // by itself) and takes 0.713 ms at 128^3, 1.16 ms before; a D2Q9 step at 128^2 4.8 us, 11.1 us before
@@ -87,8 +96,14 @@ __device__ __forceinline__ double relax_cell_f64(const double *df, const RelaxF6
     emit(0, fma(k.keep, d0, t0));
     double ksum = 0.0;  // twice the sum
     Fraction part = {0.0, 1.0};
-    if (MODE != 0) part = {fabs(fma(k.neg_tau2, t0, 2.0 * d0)), fma(k.tau, t0, w0)};
+    double n_of[2 * GROUP + 1], e_of[2 * GROUP + 1];  // the group's |n|, e; the rest's with the first
     int held = 0;
+    bool mid = true;
+    if (MODE != 0) {
+        part = {fabs(fma(k.neg_tau2, t0, 2.0 * d0)), fma(k.tau, t0, w0)};
+        n_of[held] = part.num, e_of[held++] = part.den;
+        mid = mid_range(part.den);
+    }
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
         const int o = L::opp(i);
@@ -115,9 +130,17 @@ __device__ __forceinline__ double relax_cell_f64(const double *df, const RelaxF6
             const double e = fma(k.tau, t, w), eo = k.tau * cj;
             const double np = ns + nm, nn = ns - nm, ep = e + eo, en = e - eo;
             const Fraction two = {fma(fabs(np), en, fabs(nn) * ep), ep * en};
-            part = held == 0 && i != 1 ? two : part + two;
-            if (++held == GROUP) {
-                ksum += part.num / part.den;
+            part = held == 0 ? two : part + two;
+            mid = (held == 0 || mid) && mid_range(two.den);
+            n_of[held] = fabs(np), e_of[held++] = ep;
+            n_of[held] = fabs(nn), e_of[held++] = en;
+            if (held >= 2 * GROUP) {
+                if (mid && is_finite(part.num)) {
+                    ksum += part.num / part.den;
+                } else {
+#pragma unroll
+                    for (int a = 0; a < held; ++a) ksum += n_of[a] / e_of[a];
+                }
                 held = 0;
             }
         }

@@ -272,3 +272,20 @@ def test_fp64_nan_maxima_stand_out(L, q, dims, c5, value):  # noqa: F811
     assert np.array_equal(maxima[1][~hit], maxima[0][~hit])
     assert lat.flag(1e300, block=8).reshape(hit.shape)[hit] > 0
     lat.close()
+
+
+@pytest.mark.parametrize("scale", [1e50, 1e90, 1e140])
+@pytest.mark.parametrize("q,dims", [(9, (128, 33, 1)), (19, (33, 9, 17))])
+def test_fp64_sensor_at_any_density(L, q, dims, scale):  # noqa: F811
+    """K does not change with the scale of the populations, however far their products of several are out
+    of range.  The tolerance is that of test_fp64_pairwise_relaxation."""
+    o = O.Oracle(q, *dims, tau=0.83, lid=(0.0, 0.0, 0.0))
+    f = scale * perturbed(o, seed=19, amp=0.02)
+    lat = L.Lattice(q, *dims, 0.83, dtype=L.LBM_F64, lid=(0.0, 0.0))
+    lat.set_populations(f)
+    L.lbm_set_sensor_field(lat.h, 1)
+    lat.step(1)
+    _, K, _, _ = o.step(f, sensor=True)
+    assert np.isfinite(K).all()
+    assert rel(lat.sensor_field(), K) <= 1e-12
+    lat.close()
