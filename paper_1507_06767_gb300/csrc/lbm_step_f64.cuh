@@ -81,17 +81,20 @@ __device__ __forceinline__ double relax_cell_f64(const double *df, const RelaxF6
         if (L::cy(i)) j[1] += double(L::cy(i)) * m[i];
         if (L::cz(i)) j[2] += double(L::cz(i)) * m[i];
     }
+    // the scaled momentum j = 3 omega w rho u, w the diagonal weight, and v = kappa j with kappa =
+    // 1 / (2 omega w rho): 4.5 omega w (c.j)^2 / rho is (c.j)(c.v) of these.  v is of the order of u, so no
+    // product leaves the range where the populations do not.  The term in j.j takes the same factors,
+    // so that the two cancel in the mass as far as they are rounded.
     const double inv_rho = 1.0 / (1.0 + drho);
-    double jj = 0.0;  // of the scaled momentum 3 omega w j, w the diagonal weight
+    const double kappa = k.kappa * inv_rho;
+    double jj = 0.0, v[3] = {0.0, 0.0, 0.0};
 #pragma unroll
     for (int d = 0; d < L::D; ++d) {
         j[d] = fma(j[d], k.lam, j[d] * k.lam_lo);
-        jj = fma(j[d], j[d], jj);
+        v[d] = kappa * j[d];
+        jj = fma(v[d], j[d], jj);
     }
-    // 4.5 omega w (c.j)^2 / rho = kappa (3 omega w c.j)^2 with kappa = 1 / (2 omega w rho); the term
-    // in j.j takes the same factors, so that the two cancel in the mass as far as they are rounded
-    const double kappa_d = k.kappa * inv_rho;
-    const double bd = fma(kappa_d * (-1.0 / 3.0), jj, k.feq * drho);
+    const double bd = fma(-1.0 / 3.0, jj, k.feq * drho);
     const double t0 = double(L::w36(0)) * bd;
     emit(0, fma(k.keep, d0, t0));
     double ksum = 0.0;  // twice the sum
@@ -110,17 +113,18 @@ __device__ __forceinline__ double relax_cell_f64(const double *df, const RelaxF6
         if (o < i) continue;
         const double w = weight<L, double>(i);
         const double r = double(L::w36(i));  // the weight in diagonal weights: 1, axes 4 or 2
-        double cj = 0.0;                     // 3 omega w c.j
+        double cj = 0.0, cv = 0.0;           // 3 omega w c.j
         bool first = true;
 #pragma unroll
         for (int d = 0; d < L::D; ++d) {
             const int c = d == 0 ? L::cx(i) : d == 1 ? L::cy(i) : L::cz(i);
             if (!c) continue;
             cj = first ? double(c) * j[d] : cj + double(c) * j[d];
+            cv = first ? double(c) * v[d] : cv + double(c) * v[d];
             first = false;
         }
         cj *= r;
-        const double t = fma(cj * cj, kappa_d * (1.0 / r), r * bd);
+        const double t = fma(cj, cv, r * bd);
         const double S = fma(k.half_keep, s[i], t), M = fma(k.half_keep, m[i], cj);
         emit(i, S + M);
         emit(o, S - M);

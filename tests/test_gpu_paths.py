@@ -289,3 +289,21 @@ def test_fp64_sensor_at_any_density(L, q, dims, scale):  # noqa: F811
     assert np.isfinite(K).all()
     assert rel(lat.sensor_field(), K) <= 1e-12
     lat.close()
+
+
+@pytest.mark.parametrize("scale", [1e160, 1e300])
+@pytest.mark.parametrize("q,dims", [(9, (128, 33, 1)), (19, (33, 9, 17))])
+def test_fp64_populations_at_any_density(L, q, dims, scale):  # noqa: F811
+    """No square of a momentum leaves the range before its populations do.  Tolerances as in
+    test_fp64_pairwise_relaxation."""
+    o = O.Oracle(q, *dims, tau=0.83, lid=(0.0, 0.0, 0.0))
+    f = scale * perturbed(o, seed=23, amp=0.02)
+    lat = L.Lattice(q, *dims, 0.83, dtype=L.LBM_F64, lid=(0.0, 0.0))
+    lat.set_populations(f)
+    L.lbm_set_sensor_field(lat.h, 1)
+    lat.step(3)  # two plain steps and a sensor step
+    for _ in range(3):
+        f, K, _, _ = o.step(f, sensor=True)
+    assert rel(lat.populations(), f) <= 1e-14
+    assert rel(lat.sensor_field(), K) <= 1e-12
+    lat.close()
