@@ -86,9 +86,18 @@ def pairs(feats, kmax):
 def train(net, X, T, epochs: int, batch: int, lr: float, seed: int):
     """Adam on shuffled minibatches; returns the per-epoch mean losses.  The order of the samples
     is drawn on the host from a seeded generator; an epoch is one call, whose steps read their
-    minibatches from X and T where they lie."""
+    minibatches from X [n, channels, h, w] and T (n rows of h x w) where they lie."""
     import torch
 
+    # the call knows X and T by address and n, h, w alone
+    if X.dim() != 4 or len(X) < 1 or len(T) < 1 or X.dtype != torch.float32 or T.dtype != torch.float32:
+        raise ValueError("X must be [n, channels, h, w] and T its n targets, n >= 1, both float32")
+    if T.numel() < X.shape[0] * X.shape[2] * X.shape[3]:
+        raise ValueError("T has fewer targets than X has rows")
+    if X.shape[1] != net.cin:
+        raise ValueError(f"X has {X.shape[1]} channels, the network {net.cin}")
+    if batch < 1:
+        raise ValueError("batch must be >= 1")
     g = np.random.default_rng(np.random.SeedSequence(seed))
     n, (h, w) = X.shape[0], X.shape[-2:]
     losses = []
