@@ -116,7 +116,7 @@ def step_kernel_of(w, variant="auto"):
                                                  and cells >= 1 << 17)):
         return pair
     if w["dtype"] == "F64":
-        # the one-cell kernel with the FP64 relaxation (fused_step_f64_kernel)
+        # the one-cell kernel with the FP64 relaxation (namespace lbm::f64)
         return "fused_step_kernel", ("lbm_step_f64.cuh", "lbm_step.cuh", "lbm_traits.cuh")
     return "fused_step_kernel", ("lbm_step.cuh", "lbm_traits.cuh")
 

@@ -154,16 +154,17 @@ __device__ __forceinline__ double relax_cell_f64(const double *df, const RelaxF6
 
 constexpr int F64_SPREAD_CTAS = 512;  // CTAs wanted of a plain step on a small 2-D lattice (152 SMs)
 
-// MODE, HALO and FLAT as in fused_step_kernel.  A CTA covers whole tiles as there where the step records
+namespace f64 {  // by the name of the other types' one-cell kernel: a profile lists the FP64 step with them
+
+// MODE, HALO and FLAT as in lbm::fused_step_kernel.  A CTA covers whole tiles as there where the step records
 // the tile maxima; a plain step takes one plane a CTA in 3-D and, on small 2-D lattices, fewer rows
 // (blockDim.y), as it is bound by the FP64 units: short CTAs shorten the last wave (128^3: 0.716 ms a
 // step against 0.724 with two planes and 0.737 with four) and reach every SM (128^2: 512 CTAs of one
 // row, 64 of eight).  The planes' CTAs come in a line, as there may be more than a grid's z takes.
 template <class L, int MODE, bool HALO, bool FLAT = false>
 __global__ void __launch_bounds__(CTA_X *CTA_Y, 2)
-    fused_step_f64_kernel(const double *__restrict__ fin, double *__restrict__ fout,
-                          StepParams p, double *__restrict__ tile_max,
-                          double *__restrict__ k_field, const RelaxF64 k) {
+    fused_step_kernel(const double *__restrict__ fin, double *__restrict__ fout, StepParams p,
+                      double *__restrict__ tile_max, double *__restrict__ k_field, const RelaxF64 k) {
     constexpr int Q = L::Q;
     constexpr int ZT = MODE != 0 && L::D == 3 ? TILE : 1;
     const int nx = p.nx, ny = p.ny, nz = p.nz;
@@ -235,6 +236,8 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, 2)
     }
 }
 
+}  // namespace f64
+
 template <class L, bool HALO = false>
 cudaError_t launch_fused_step_f64(const void *fin, void *fout, const StepParams &p, int mode,
                                   void *tile_max, void *k_field, cudaStream_t stream) {
@@ -252,15 +255,15 @@ cudaError_t launch_fused_step_f64(const void *fin, void *fout, const StepParams 
     if constexpr (!HALO) {
         if (mode == 0 && flat_rows<L>(p, mode, 0, 1)) {
             grid.x = (unsigned)(((long long)p.nx * p.ny + CTA_X * rows - 1) / (CTA_X * rows) * gz);
-            return launch_step_kernel<L>(fused_step_f64_kernel<L, 0, false, true>, grid, block, 0,
+            return launch_step_kernel<L>(f64::fused_step_kernel<L, 0, false, true>, grid, block, 0,
                                          stream, a, b, p, tm, kf, k);
         }
     }
     if (mode == 0)
-        return launch_step_kernel<L>(fused_step_f64_kernel<L, 0, HALO>, grid, block, 0, stream, a, b, p, tm, kf, k);
+        return launch_step_kernel<L>(f64::fused_step_kernel<L, 0, HALO>, grid, block, 0, stream, a, b, p, tm, kf, k);
     if (mode == 1)
-        return launch_step_kernel<L>(fused_step_f64_kernel<L, 1, HALO>, grid, block, 0, stream, a, b, p, tm, kf, k);
-    return launch_step_kernel<L>(fused_step_f64_kernel<L, 2, HALO>, grid, block, 0, stream, a, b, p, tm, kf, k);
+        return launch_step_kernel<L>(f64::fused_step_kernel<L, 1, HALO>, grid, block, 0, stream, a, b, p, tm, kf, k);
+    return launch_step_kernel<L>(f64::fused_step_kernel<L, 2, HALO>, grid, block, 0, stream, a, b, p, tm, kf, k);
 }
 
 }  // namespace lbm

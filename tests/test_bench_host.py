@@ -141,3 +141,11 @@ def test_clock_sampler_without_samples():
     assert s.stop() is None  # never started
     s.proc, s.thread, s.lines = _Proc(), _Thread(), []
     assert s.stop() is None
+
+
+@pytest.mark.parametrize("workload", ["d3q19_256_fp32_re1000", "d3q19_512_f16s_re1000", "d2q9_128_fp64_re100",
+                                      "d2q9_1024_learned"])
+def test_the_named_step_kernel_is_defined_where_it_says(workload):
+    name, headers = bench.step_kernel_of(bench.WORKLOADS[workload])
+    src = open(os.path.join(bench.ROOT, "paper_1507_06767_gb300", "csrc", headers[0])).read()
+    assert f" {name}(const " in src.replace("\n", " ")
