@@ -449,14 +449,16 @@ cudaError_t launch_fused_step(const void *fin, void *fout, const StepParams &p, 
     T *b = static_cast<T *>(fout);
     R *tm = static_cast<R *>(tile_max);
     R *kf = static_cast<R *>(k_field);
-    if constexpr (!HALO && DT != 0) {
+    if constexpr (!HALO && (L::D == 3 || DT == 1)) {  // the types and modes that flat_rows takes
         if (flat_rows<L>(p, mode, DT, 1)) {
             grid.x = (unsigned)(((long long)p.nx * p.ny + CTA_X * CTA_Y - 1) / (CTA_X * CTA_Y));
             grid.y = 1;
-            return launch_step_kernel<L>(mode == 0   ? fused_step_kernel<L, DT, 0, false, true>
-                                         : mode == 1 ? fused_step_kernel<L, DT, 1, false, true>
-                                                     : fused_step_kernel<L, DT, 2, false, true>,
-                                         grid, block, 0, stream, a, b, p, tm, kf);
+            auto *kernel = fused_step_kernel<L, DT, 0, false, true>;
+            if constexpr (L::D == 3)
+                kernel = mode == 0   ? kernel
+                         : mode == 1 ? fused_step_kernel<L, DT, 1, false, true>
+                                     : fused_step_kernel<L, DT, 2, false, true>;
+            return launch_step_kernel<L>(kernel, grid, block, 0, stream, a, b, p, tm, kf);
         }
     }
     if (mode == 0)

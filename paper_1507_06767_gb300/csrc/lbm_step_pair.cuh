@@ -378,11 +378,13 @@ cudaError_t launch_fused_step_pair(const void *fin, void *fout, const StepParams
     T *b = static_cast<T *>(fout);
     float *tm = static_cast<float *>(tile_max);
     float *kf = static_cast<float *>(k_field);
-    if (flat_rows<L>(p, mode, DT, 2)) {
-        grid.x = FlatLine(p.nx / 2, p.ny).ctas(CTA_X * CTA_Y);
-        grid.y = 1;
-        return launch_step_kernel<L>(fused_step_pair_kernel<L, DT, 0, true>, grid, block, 0, stream, a,
-                                     b, p, tm, kf);
+    if constexpr (L::D == 3) {
+        if (flat_rows<L>(p, mode, DT, 2)) {
+            grid.x = FlatLine(p.nx / 2, p.ny).ctas(CTA_X * CTA_Y);
+            grid.y = 1;
+            return launch_step_kernel<L>(fused_step_pair_kernel<L, DT, 0, true>, grid, block, 0, stream,
+                                         a, b, p, tm, kf);
+        }
     }
     if (mode == 0)
         return launch_step_kernel<L>(fused_step_pair_kernel<L, DT, 0>, grid, block, 0, stream, a, b, p, tm, kf);
