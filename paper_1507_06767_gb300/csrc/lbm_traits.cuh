@@ -106,11 +106,10 @@ struct Storage<3> {  // LBM_BF16S
 // Order-preserving integer image of a non-negative-or-NaN value, used for max reductions:
 // for K >= 0 the bit pattern orders like the value, and a (positive) NaN beats every finite value
 // and +inf, so a NaN in a tile poisons its maximum.  FP32 arithmetic gives the positive NaN; in FP64
-// an invalid operation gives the negative one, whose sign is dropped here.
+// an invalid operation gives the negative one, so any NaN is taken as the positive one.
 __device__ __forceinline__ int max_bits(float v) { return __float_as_int(v); }
 __device__ __forceinline__ long long max_bits(double v) {
-    const long long b = __double_as_longlong(v), a = b & 0x7fffffffffffffffll;
-    return a > 0x7ff0000000000000ll ? a : b;
+    return v != v ? 0x7ff8000000000000ll : __double_as_longlong(v);
 }
 __device__ __forceinline__ float from_bits(int b, float) { return __int_as_float(b); }
 __device__ __forceinline__ double from_bits(long long b, double) { return __longlong_as_double(b); }
