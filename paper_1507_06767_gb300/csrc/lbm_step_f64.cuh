@@ -53,16 +53,19 @@ __device__ __forceinline__ bool is_finite(double v) {
 //     M = (1 - omega) / 2 m + 3 omega w c.j,   B = rho - 1 - 1.5 j.j / rho,
 // where j = rho u.  The momentum is scaled once by 3 omega w (w the diagonal weight), so that c.j is
 // one addition in both S and M.  The sensor's fractions |f^neq| / f^eq are added over common
-// denominators, three opposite pairs (two in 2-D) to one division.  Where a pair's product of equilibria
-// is far from one (densities beyond 1e45, zeros, infinities, NaN) or the numerator overflows, that
-// group's fractions are divided one by one, as the products of three pairs would leave the range.
+// denominators, three opposite pairs (two in 2-D) to one division.  mid (MODE != 0) comes back false
+// where a pair's product of equilibria is so far from one that a product of three may leave the range
+// (densities beyond 1e45, zeros, infinities, NaN) or a numerator overflows: the sensor is then
+// sensor_cell_f64's.  That one gathers the cell again; kept at hand for it, the fractions took the 2-D
+// kernel from 64 to 76 registers and a sensor step of 301 x 203 from 23.8 to 34.6 us.
 //
 // A plain D3Q19 step issues about 165 FP64 instructions a cell (about 350 with each direction relaxed
 // by itself) and takes 0.713 ms at 128^3, 1.16 ms before; a D2Q9 step at 128^2 4.8 us, 11.1 us before
 // (with the smaller CTAs below).  After 100 steps of a 128^2 cavity the populations are 0.5e-16 to
 // 1.3e-16 off an 80-bit evaluation, 2.2e-16 to 2.7e-16 before.
 template <class L, int MODE, class Emit>
-__device__ __forceinline__ double relax_cell_f64(const double *df, const RelaxF64 &k, Emit &&emit) {
+__device__ __forceinline__ double relax_cell_f64(const double *df, const RelaxF64 &k, bool &mid,
+                                                 Emit &&emit) {
     constexpr int Q = L::Q;
     constexpr int GROUP = L::D == 3 ? 3 : 2;
     static_assert((Q - 1) / 2 % GROUP == 0, "whole groups of pairs");
@@ -99,14 +102,11 @@ __device__ __forceinline__ double relax_cell_f64(const double *df, const RelaxF6
     emit(0, fma(k.keep, d0, t0));
     double ksum = 0.0;  // twice the sum
     Fraction part = {0.0, 1.0};
-    double n_of[2 * GROUP + 1], e_of[2 * GROUP + 1];  // the group's |n|, e; the rest's with the first
-    int held = 0;
-    bool mid = true;
     if (MODE != 0) {
         part = {fabs(fma(k.neg_tau2, t0, 2.0 * d0)), fma(k.tau, t0, w0)};
-        n_of[held] = part.num, e_of[held++] = part.den;
         mid = mid_range(part.den);
     }
+    int held = 0;
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
         const int o = L::opp(i);
@@ -134,22 +134,41 @@ __device__ __forceinline__ double relax_cell_f64(const double *df, const RelaxF6
             const double e = fma(k.tau, t, w), eo = k.tau * cj;
             const double np = ns + nm, nn = ns - nm, ep = e + eo, en = e - eo;
             const Fraction two = {fma(fabs(np), en, fabs(nn) * ep), ep * en};
-            part = held == 0 ? two : part + two;
-            mid = (held == 0 || mid) && mid_range(two.den);
-            n_of[held] = fabs(np), e_of[held++] = ep;
-            n_of[held] = fabs(nn), e_of[held++] = en;
-            if (held >= 2 * GROUP) {
-                if (mid && is_finite(part.num)) {
-                    ksum += part.num / part.den;
-                } else {
-#pragma unroll
-                    for (int a = 0; a < held; ++a) ksum += n_of[a] / e_of[a];
-                }
+            part = held == 0 && i != 1 ? two : part + two;
+            mid = mid && mid_range(two.den);
+            if (++held == GROUP) {
+                mid = mid && is_finite(part.num);
+                ksum += part.num / part.den;
                 held = 0;
             }
         }
     }
     return ksum * (0.5 / double(Q));
+}
+
+// The sensor of one cell, each fraction divided by itself.
+template <class L>
+__device__ __forceinline__ double sensor_cell_f64(const double *df) {
+    double drho = 0.0, u[3] = {0.0, 0.0, 0.0}, uu = 0.0, ksum = 0.0;
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) {
+        drho += df[i];
+        u[0] += double(L::cx(i)) * df[i];
+        u[1] += double(L::cy(i)) * df[i];
+        u[2] += double(L::cz(i)) * df[i];
+    }
+    const double rho = 1.0 + drho, inv_rho = 1.0 / rho;
+    for (int d = 0; d < 3; ++d) {
+        u[d] *= inv_rho;
+        uu = fma(u[d], u[d], uu);
+    }
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i) {
+        const double cu = double(L::cx(i)) * u[0] + double(L::cy(i)) * u[1] + double(L::cz(i)) * u[2];
+        const double P = fma(4.5 * cu, cu, fma(3.0, cu, -1.5 * uu)), w = weight<L, double>(i);
+        ksum += fabs(df[i] - w * fma(rho, P, drho)) / (w * rho * (1.0 + P));
+    }
+    return ksum * (1.0 / double(L::Q));
 }
 
 constexpr int F64_SPREAD_CTAS = 512;  // CTAs wanted of a plain step on a small 2-D lattice (152 SMs)
@@ -162,7 +181,7 @@ namespace f64 {  // by the name of the other types' one-cell kernel: a profile l
 // step against 0.724 with two planes and 0.737 with four) and reach every SM (128^2: 512 CTAs of one
 // row, 64 of eight).  The planes' CTAs come in a line, as there may be more than a grid's z takes.
 template <class L, int MODE, bool HALO, bool FLAT = false>
-__global__ void __launch_bounds__(CTA_X *CTA_Y, 2)
+__global__ void __launch_bounds__(CTA_X *CTA_Y, L::D == 2 ? 4 : 2)
     fused_step_kernel(const double *__restrict__ fin, double *__restrict__ fout, StepParams p,
                       double *__restrict__ tile_max, double *__restrict__ k_field, const RelaxF64 k) {
     constexpr int Q = L::Q;
@@ -206,10 +225,15 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, 2)
             gather_xsel<L, 0>(fin, N, nx, nx * ny, (size_t)idx, x, p.periodic & 1, df);
         else
             gather_cell<L, 0, 1, HALO>(fin, p, N, x, y, z, df);
-        const double K = relax_cell_f64<L, MODE>(df, k, [&](int i, double d) {
+        bool mid;
+        double K = relax_cell_f64<L, MODE>(df, k, mid, [&](int i, double d) {
             fout[(size_t)i * N + idx] = d + weight<L, double>(i);
         });
         if (MODE != 0) {
+            if (!mid) {
+                gather_cell<L, 0, 1, HALO>(fin, p, N, x, y, z, df);
+                K = sensor_cell_f64<L>(df);
+            }
             const long long kb = max_bits(K);
             kmax = kb > kmax ? kb : kmax;
             if (MODE == 2) k_field[idx] = K;
