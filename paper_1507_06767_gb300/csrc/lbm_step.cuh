@@ -15,6 +15,8 @@
 // without cancelling against w_i.
 #pragma once
 
+#include <atomic>
+
 #include "lbm_internal.h"
 
 namespace lbm {
@@ -288,7 +290,14 @@ __device__ __forceinline__ typename Storage<DT>::R relax_store_cell(
     });
 }
 
-// The halo planes are read behind pdl_wait too: the launch before the step may have filled them.
+// Wait for the step before a 2-D step (launch_step_kernel).  The next one may start from here or, LATE,
+// where the kernel says so at its end.
+template <bool LATE, class T>
+__device__ __forceinline__ T *step_wait(T *fin) {
+    return LATE ? pdl_wait_only(fin) : pdl_wait(fin);
+}
+
+// The halo planes are read behind the wait too: the launch before the step may have filled them.
 __device__ __forceinline__ void order_halos(StepParams &p) {
     p.halo_lo = pdl_order(p.halo_lo);
     p.halo_hi = pdl_order(p.halo_hi);
@@ -305,8 +314,9 @@ __device__ __forceinline__ void combine_tile_max(int tile, int kmax, float *tile
 // MODE 0: no sensor.  MODE 1: sensor and per-tile max.  MODE 2: MODE 1 plus per-cell K.  HALO:
 // the faces of the slowest axis may be cuts of a slab (gather_cell).  FLAT (no halo): a CTA takes 256
 // consecutive cells of a plane, wherever rows begin and end among them; CTAs share tiles then, whose
-// maxima they combine with atomics in a buffer that the sensor step before has cleared.
-template <class L, int DT, int MODE, bool HALO = false, bool FLAT = false>
+// maxima they combine with atomics in a buffer that the sensor step before has cleared.  LATE (2-D): see
+// launch_step_kernel.
+template <class L, int DT, int MODE, bool HALO = false, bool FLAT = false, bool LATE = false>
 __global__ void __launch_bounds__(CTA_X *CTA_Y, LBM_STEP_MIN_BLOCKS)
     fused_step_kernel(const typename Storage<DT>::T *__restrict__ fin,
                       typename Storage<DT>::T *__restrict__ fout, StepParams p,
@@ -329,7 +339,7 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, LBM_STEP_MIN_BLOCKS)
     const size_t N = (size_t)nx * ny * nz;
     const R omega = param_omega<R>(p);
 
-    if constexpr (L::D == 2) fin = pdl_wait(fin);
+    if constexpr (L::D == 2) fin = step_wait<LATE>(fin);
     if constexpr (L::D == 2 && HALO) order_halos(p);
 
     // clear the other tile buffer for the next sensor step (kernels that combine tiles across
@@ -375,6 +385,7 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, LBM_STEP_MIN_BLOCKS)
         }
     }
 
+    if constexpr (LATE) pdl_start_next();
     if constexpr (FLAT && MODE != 0)
         combine_tile_max(active ? (blockIdx.z * p.nty + y / TILE) * p.ntx + x / TILE : -1, kmax,
                          tile_max);
@@ -401,15 +412,60 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, LBM_STEP_MIN_BLOCKS)
     }
 }
 
+// CTAs of a kernel that one SM and the GPU hold, asked for once.
+struct Resident {
+    int per_sm, all;
+};
+template <auto KERNEL>
+inline Resident resident_ctas(int threads) {
+    static std::atomic<int> known[CTA_Y + 1];  // by warps; 0: not asked yet
+    static std::atomic<int> sms{0};
+    const int warps = threads / CTA_X;
+    int n = known[warps].load(std::memory_order_relaxed), m = sms.load(std::memory_order_relaxed);
+    if (n == 0 || m == 0) {
+        int dev = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, KERNEL, threads, 0) != cudaSuccess ||
+            cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&m, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            return {0, 0};
+        known[warps].store(n, std::memory_order_relaxed);
+        sms.store(m, std::memory_order_relaxed);
+    }
+    return {n, n * m};
+}
+
 // Launch of a step kernel.  In 2-D, where a step may take a few us, it overlaps its start with the
-// end of the step before (launch_pdl): 128^2 FP64 4.95 -> 4.80 us a step.  In 3-D the CTAs that wait
-// take the place of running ones: 195 x 129 x 97 FP32 78.0 -> 79.7 us, so not there.
-template <class L, class... Params, class... Args>
-inline cudaError_t launch_step_kernel(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem,
-                                      cudaStream_t s, Args... args) {
-    if (L::D == 2) return launch_pdl(kernel, grid, block, smem, s, args...);
-    kernel<<<grid, block, smem, s>>>(args...);
-    return cudaGetLastError();
+// end of the step before (launch_pdl): 128^2 FP64 4.62 -> 4.49 us a step in a graph, 6.16 -> 4.52 in calls
+// of one step, 4096^2 FP32 170.9 either way.  In 3-D the CTAs that wait take the place of running ones:
+// 195 x 129 x 97 FP32 78.0 -> 79.7 us, so not there.
+//
+// Waiting CTAs also settle where the step before has left room.  Where the GPU holds one step but not two, and
+// one does not fill it, the next step's CTAs then lie unevenly over the SMs, up to the most an SM takes.
+// So such a step (LATE) lets the next one start at the end of its CTAs: 320^2 FP64 27.6 -> 19.1 us (19.3 without
+// overlap), with the sensor 45.5 -> 34.6 (36.9); 448^2 FP32 3.22 -> 2.83 (3.08), FP16 3.15 -> 2.70 (2.83).
+// Elsewhere the early start gains: 480^2 FP32 3.47 -> 3.21, 900^2 FP16 6.07 -> 5.83, 1025 x 1023 FP16
+// 10.68 -> 9.77; but not in FP64, which is always late.  Two kernels, as one that chooses at run time
+// schedules its stores ahead of the choice and loses as much in FP32 and 16 bits.
+template <class L, auto EARLY, auto LATE, class... Args>
+inline cudaError_t launch_step_kernel(dim3 grid, dim3 block, cudaStream_t s, Args... args) {
+    if constexpr (L::D == 3) {
+        EARLY<<<grid, block, 0, s>>>(args...);
+        return cudaGetLastError();
+    } else {
+        bool late = true;
+        if constexpr (EARLY != LATE) {
+            const Resident r = resident_ctas<EARLY>(block.x * block.y);
+            const long long ctas = (long long)grid.x * grid.y;
+            late = r.per_sm > 0 && 2 * ctas > r.all && ctas <= r.all - r.all / r.per_sm;
+        }
+        return launch_pdl(late ? LATE : EARLY, grid, block, 0, s, args...);
+    }
+}
+
+template <class L, int DT, int MODE, bool HALO, bool FLAT, class... Args>
+inline cudaError_t launch_step(dim3 grid, dim3 block, cudaStream_t s, Args... args) {
+    return launch_step_kernel<L, fused_step_kernel<L, DT, MODE, HALO, FLAT>,
+                              fused_step_kernel<L, DT, MODE, HALO, FLAT, L::D == 2>>(grid, block, s, args...);
 }
 
 // Whether a step takes the cells of a plane in a line (FLAT) rather than in rows of CTA_X lanes; dtype
@@ -453,19 +509,20 @@ cudaError_t launch_fused_step(const void *fin, void *fout, const StepParams &p, 
         if (flat_rows<L>(p, mode, DT, 1)) {
             grid.x = (unsigned)(((long long)p.nx * p.ny + CTA_X * CTA_Y - 1) / (CTA_X * CTA_Y));
             grid.y = 1;
-            auto *kernel = fused_step_kernel<L, DT, 0, false, true>;
-            if constexpr (L::D == 3)
-                kernel = mode == 0   ? kernel
-                         : mode == 1 ? fused_step_kernel<L, DT, 1, false, true>
-                                     : fused_step_kernel<L, DT, 2, false, true>;
-            return launch_step_kernel<L>(kernel, grid, block, 0, stream, a, b, p, tm, kf);
+            if constexpr (L::D == 3) {
+                if (mode == 1)
+                    return launch_step<L, DT, 1, false, true>(grid, block, stream, a, b, p, tm, kf);
+                if (mode == 2)
+                    return launch_step<L, DT, 2, false, true>(grid, block, stream, a, b, p, tm, kf);
+            }
+            return launch_step<L, DT, 0, false, true>(grid, block, stream, a, b, p, tm, kf);
         }
     }
     if (mode == 0)
-        return launch_step_kernel<L>(fused_step_kernel<L, DT, 0, HALO>, grid, block, 0, stream, a, b, p, tm, kf);
+        return launch_step<L, DT, 0, HALO, false>(grid, block, stream, a, b, p, tm, kf);
     if (mode == 1)
-        return launch_step_kernel<L>(fused_step_kernel<L, DT, 1, HALO>, grid, block, 0, stream, a, b, p, tm, kf);
-    return launch_step_kernel<L>(fused_step_kernel<L, DT, 2, HALO>, grid, block, 0, stream, a, b, p, tm, kf);
+        return launch_step<L, DT, 1, HALO, false>(grid, block, stream, a, b, p, tm, kf);
+    return launch_step<L, DT, 2, HALO, false>(grid, block, stream, a, b, p, tm, kf);
 }
 
 // A slab with halo faces (StepParams::halo_lo / halo_hi) runs the one-cell kernel with the halo

@@ -217,7 +217,7 @@ struct FlatLine {
 };
 
 // FLAT (MODE 0): the pairs of a plane in the order of FlatLine rather than in rows of 32 lanes.
-template <class L, int DT, int MODE, bool FLAT = false>
+template <class L, int DT, int MODE, bool FLAT = false, bool LATE = false>
 __global__ void __launch_bounds__(CTA_X *CTA_Y, DT == 1 ? LBM_PAIR_MIN_BLOCKS_F32 : LBM_PAIR_MIN_BLOCKS)
     fused_step_pair_kernel(const typename Storage<DT>::T *__restrict__ fin,
                            typename Storage<DT>::T *__restrict__ fout, const StepParams p,
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, DT == 1 ? LBM_PAIR_MIN_BLOCKS_F3
     const unsigned nxy = (unsigned)nx * (unsigned)ny;
 
     int kmax = 0;
-    if constexpr (L::D == 2) fin = pdl_wait(fin);
+    if constexpr (L::D == 2) fin = step_wait<LATE>(fin);
 
     if (MODE != 0 && p.tile_zero) {
         const size_t nt = (size_t)p.ntx * p.nty * p.ntz;
@@ -334,6 +334,7 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, DT == 1 ? LBM_PAIR_MIN_BLOCKS_F3
         }
     }
 
+    if constexpr (LATE) pdl_start_next();
     if (MODE != 0) {
         // a warp row covers 64 cells = 8 tiles of 8 cells = 4 lanes per tile
 #pragma unroll
@@ -365,6 +366,12 @@ inline bool pair_applicable(const StepParams &p) {
     return p.nx % 2 == 0 && (unsigned long long)(L::Q + 1) * cells < (1ULL << 32);
 }
 
+template <class L, int DT, int MODE, bool FLAT, class... Args>
+inline cudaError_t launch_step_pair(dim3 grid, dim3 block, cudaStream_t s, Args... args) {
+    return launch_step_kernel<L, fused_step_pair_kernel<L, DT, MODE, FLAT>,
+                              fused_step_pair_kernel<L, DT, MODE, FLAT, L::D == 2>>(grid, block, s, args...);
+}
+
 template <class L, int DT>
 cudaError_t launch_fused_step_pair(const void *fin, void *fout, const StepParams &p, int mode,
                                    void *tile_max, void *k_field, cudaStream_t stream) {
@@ -382,15 +389,14 @@ cudaError_t launch_fused_step_pair(const void *fin, void *fout, const StepParams
         if (flat_rows<L>(p, mode, DT, 2)) {
             grid.x = FlatLine(p.nx / 2, p.ny).ctas(CTA_X * CTA_Y);
             grid.y = 1;
-            return launch_step_kernel<L>(fused_step_pair_kernel<L, DT, 0, true>, grid, block, 0, stream,
-                                         a, b, p, tm, kf);
+            return launch_step_pair<L, DT, 0, true>(grid, block, stream, a, b, p, tm, kf);
         }
     }
     if (mode == 0)
-        return launch_step_kernel<L>(fused_step_pair_kernel<L, DT, 0>, grid, block, 0, stream, a, b, p, tm, kf);
+        return launch_step_pair<L, DT, 0, false>(grid, block, stream, a, b, p, tm, kf);
     if (mode == 1)
-        return launch_step_kernel<L>(fused_step_pair_kernel<L, DT, 1>, grid, block, 0, stream, a, b, p, tm, kf);
-    return launch_step_kernel<L>(fused_step_pair_kernel<L, DT, 2>, grid, block, 0, stream, a, b, p, tm, kf);
+        return launch_step_pair<L, DT, 1, false>(grid, block, stream, a, b, p, tm, kf);
+    return launch_step_pair<L, DT, 2, false>(grid, block, stream, a, b, p, tm, kf);
 }
 
 }  // namespace lbm

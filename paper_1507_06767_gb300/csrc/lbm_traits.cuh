@@ -134,6 +134,16 @@ __device__ __forceinline__ T *pdl_wait(T *p) {
     return p;
 }
 
+// The two apart, for a kernel that says later that the next one may start.
+template <class T>
+__device__ __forceinline__ T *pdl_wait_only(T *p) {
+    asm volatile("griddepcontrol.wait;" : "+l"(p) : : "memory");
+    return p;
+}
+__device__ __forceinline__ void pdl_start_next() {
+    asm volatile("griddepcontrol.launch_dependents;" : : : "memory");
+}
+
 // Another pointer that is read after pdl_wait: it is not known before the wait.
 template <class T>
 __device__ __forceinline__ T *pdl_order(T *p) {

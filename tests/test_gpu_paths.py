@@ -307,3 +307,30 @@ def test_fp64_populations_at_any_density(L, q, dims, scale):  # noqa: F811
     assert rel(lat.populations(), f) <= 1e-14
     assert rel(lat.sensor_field(), K) <= 1e-12
     lat.close()
+
+
+@pytest.mark.parametrize("dtype,nx,ny", [("LBM_F64", 320, 320), ("LBM_F64", 384, 380), ("LBM_F64", 416, 416),
+                                         ("LBM_F32", 448, 448), ("LBM_F32", 480, 480), ("LBM_F32", 333, 444),
+                                         ("LBM_F16S", 448, 450), ("LBM_F16S", 900, 900)])
+def test_2d_steps_of_any_share_of_the_gpu_overlap(L, dtype, nx, ny):  # noqa: F811
+    """Steps that fill the SMs in part, just or more than once let the next one start early or late: runs,
+    with the sensor at every third step, give the bits of steps with a wait after each."""
+    import torch
+
+    o = O.Oracle(9, nx, ny, 1, tau=0.7, lid=(0.1, 0.0, 0.0))
+    f = perturbed(o, seed=nx + ny, amp=0.02)
+    lats = [L.Lattice(9, nx, ny, 1, 0.7, dtype=getattr(L, dtype), lid=(0.1, 0.0)) for _ in range(2)]
+    for lat in lats:
+        lat.set_populations(f)
+        L.lbm_set_graphs(lat.h, 0)
+    for every in (3, 1000):
+        for lat in lats:
+            L.lbm_set_sensor_every(lat.h, every)
+        lats[0].step(30)
+        for _ in range(30):
+            lats[1].step(1)
+            torch.cuda.synchronize()
+        assert np.array_equal(lats[0].raw(), lats[1].raw())
+        assert np.array_equal(lats[0].sensor(8), lats[1].sensor(8))
+    for lat in lats:
+        lat.close()
