@@ -443,21 +443,18 @@ inline Resident resident_ctas(int threads) {
 // one does not fill it, the next step's CTAs then lie unevenly over the SMs, up to the most an SM takes.
 // So such a step (LATE) lets the next one start at the end of its CTAs: 320^2 FP64 27.6 -> 19.1 us (19.3 without
 // overlap), with the sensor 45.5 -> 34.6 (36.9); 448^2 FP32 3.22 -> 2.83 (3.08), FP16 3.15 -> 2.70 (2.83).
-// Elsewhere the early start gains: 480^2 FP32 3.47 -> 3.21, 900^2 FP16 6.07 -> 5.83, 1025 x 1023 FP16
-// 10.68 -> 9.77; but not in FP64, which is always late.  Two kernels, as one that chooses at run time
-// schedules its stores ahead of the choice and loses as much in FP32 and 16 bits.
+// Elsewhere the early start gains: 128^2 FP64 4.61 -> 4.49, 480^2 FP32 3.47 -> 3.21, 900^2 FP16 6.07 ->
+// 5.83.  Two kernels, as one that chooses at run time is scheduled around the choice: 1025 x 1023 FP16
+// 9.77 -> 10.68.
 template <class L, auto EARLY, auto LATE, class... Args>
 inline cudaError_t launch_step_kernel(dim3 grid, dim3 block, cudaStream_t s, Args... args) {
     if constexpr (L::D == 3) {
         EARLY<<<grid, block, 0, s>>>(args...);
         return cudaGetLastError();
     } else {
-        bool late = true;
-        if constexpr (EARLY != LATE) {
-            const Resident r = resident_ctas<EARLY>(block.x * block.y);
-            const long long ctas = (long long)grid.x * grid.y;
-            late = r.per_sm > 0 && 2 * ctas > r.all && ctas <= r.all - r.all / r.per_sm;
-        }
+        const Resident r = resident_ctas<EARLY>(block.x * block.y);
+        const long long ctas = (long long)grid.x * grid.y;
+        const bool late = r.per_sm > 0 && 2 * ctas > r.all && ctas <= r.all - r.all / r.per_sm;
         return launch_pdl(late ? LATE : EARLY, grid, block, 0, s, args...);
     }
 }

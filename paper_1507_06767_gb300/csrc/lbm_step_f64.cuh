@@ -175,12 +175,12 @@ constexpr int F64_SPREAD_CTAS = 512;  // CTAs wanted of a plain step on a small 
 
 namespace f64 {  // by the name of the other types' one-cell kernel: a profile lists the FP64 step with them
 
-// MODE, HALO and FLAT as in lbm::fused_step_kernel.  A CTA covers whole tiles as there where the step records
+// MODE, HALO, FLAT and LATE as in lbm::fused_step_kernel.  A CTA covers whole tiles as there where the step records
 // the tile maxima; a plain step takes one plane a CTA in 3-D and, on small 2-D lattices, fewer rows
 // (blockDim.y), as it is bound by the FP64 units: short CTAs shorten the last wave (128^3: 0.716 ms a
 // step against 0.724 with two planes and 0.737 with four) and reach every SM (128^2: 512 CTAs of one
 // row, 64 of eight).  The planes' CTAs come in a line, as there may be more than a grid's z takes.
-template <class L, int MODE, bool HALO, bool FLAT = false>
+template <class L, int MODE, bool HALO, bool FLAT = false, bool LATE = false>
 __global__ void __launch_bounds__(CTA_X *CTA_Y, L::D == 3 ? 2 : MODE == 0 ? 5 : 4)
     fused_step_kernel(const double *__restrict__ fin, double *__restrict__ fout, StepParams p,
                       double *__restrict__ tile_max, double *__restrict__ k_field, const RelaxF64 k) {
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, L::D == 3 ? 2 : MODE == 0 ? 5 : 
     const int x = FLAT ? at - y * nx : bx * CTA_X + lane, z0 = bz * ZT;
     const bool active = (x < nx) && (y < ny);
     const size_t N = (size_t)nx * ny * nz;
-    if constexpr (L::D == 2) fin = step_wait<true>(fin);
+    if constexpr (L::D == 2) fin = step_wait<LATE>(fin);
     if constexpr (L::D == 2 && HALO) order_halos(p);
     if (MODE != 0 && p.tile_zero) {  // as in fused_step_kernel
         const size_t nt = (size_t)p.ntx * p.nty * p.ntz, me = (size_t)blockIdx.x * (CTA_X * CTA_Y) +
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, L::D == 3 ? 2 : MODE == 0 ? 5 : 
             if (MODE == 2) k_field[idx] = K;
         }
     }
-    if constexpr (L::D == 2) pdl_start_next();
+    if constexpr (LATE) pdl_start_next();
     if (MODE != 0) {
         // max over the 8 lanes of each x-tile of this row, then over the 8 rows via shared memory
 #pragma unroll
@@ -263,9 +263,10 @@ __global__ void __launch_bounds__(CTA_X *CTA_Y, L::D == 3 ? 2 : MODE == 0 ? 5 : 
 
 }  // namespace f64
 
-template <class L, auto KERNEL, class... Args>
-inline cudaError_t launch_f64(dim3 grid, dim3 block, cudaStream_t s, Args... args) {
-    return launch_step_kernel<L, KERNEL, KERNEL>(grid, block, s, args...);
+template <class L, int MODE, bool HALO, bool FLAT, class... Args>
+inline cudaError_t launch_step_f64(dim3 grid, dim3 block, cudaStream_t s, Args... args) {
+    return launch_step_kernel<L, f64::fused_step_kernel<L, MODE, HALO, FLAT>,
+                              f64::fused_step_kernel<L, MODE, HALO, FLAT, L::D == 2>>(grid, block, s, args...);
 }
 
 template <class L, bool HALO = false>
@@ -285,14 +286,14 @@ cudaError_t launch_fused_step_f64(const void *fin, void *fout, const StepParams 
     if constexpr (!HALO) {
         if (mode == 0 && flat_rows<L>(p, mode, 0, 1)) {
             grid.x = (unsigned)(((long long)p.nx * p.ny + CTA_X * rows - 1) / (CTA_X * rows) * gz);
-            return launch_f64<L, f64::fused_step_kernel<L, 0, false, true>>(grid, block, stream, a, b, p, tm, kf, k);
+            return launch_step_f64<L, 0, false, true>(grid, block, stream, a, b, p, tm, kf, k);
         }
     }
     if (mode == 0)
-        return launch_f64<L, f64::fused_step_kernel<L, 0, HALO>>(grid, block, stream, a, b, p, tm, kf, k);
+        return launch_step_f64<L, 0, HALO, false>(grid, block, stream, a, b, p, tm, kf, k);
     if (mode == 1)
-        return launch_f64<L, f64::fused_step_kernel<L, 1, HALO>>(grid, block, stream, a, b, p, tm, kf, k);
-    return launch_f64<L, f64::fused_step_kernel<L, 2, HALO>>(grid, block, stream, a, b, p, tm, kf, k);
+        return launch_step_f64<L, 1, HALO, false>(grid, block, stream, a, b, p, tm, kf, k);
+    return launch_step_f64<L, 2, HALO, false>(grid, block, stream, a, b, p, tm, kf, k);
 }
 
 }  // namespace lbm
