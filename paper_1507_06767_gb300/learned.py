@@ -90,16 +90,16 @@ def train(net, X, T, epochs: int, batch: int, lr: float, seed: int):
     import torch
 
     # the call knows X and T by address and n, h, w alone
-    if X.dim() != 4 or len(X) < 1 or len(T) < 1 or X.dtype != torch.float32 or T.dtype != torch.float32:
-        raise ValueError("X must be [n, channels, h, w] and T its n targets, n >= 1, both float32")
-    if T.numel() < X.shape[0] * X.shape[2] * X.shape[3]:
-        raise ValueError("T has fewer targets than X has rows")
-    if X.shape[1] != net.cin:
-        raise ValueError(f"X has {X.shape[1]} channels, the network {net.cin}")
+    if X.dim() != 4 or X.dtype != torch.float32 or T.dtype != torch.float32:
+        raise ValueError("X must be [n, channels, h, w], X and T float32")
+    n, channels, h, w = X.shape
+    if n < 1 or T.numel() < n * h * w:
+        raise ValueError("X must have rows and T as many targets")
+    if channels != net.cin:
+        raise ValueError(f"X has {channels} channels, the network {net.cin}")
     if batch < 1:
         raise ValueError("batch must be >= 1")
     g = np.random.default_rng(np.random.SeedSequence(seed))
-    n, (h, w) = X.shape[0], X.shape[-2:]
     losses = []
     for _ in range(epochs):
         perm = torch.from_numpy(g.permutation(n).astype(np.int32)).cuda()
