@@ -82,6 +82,8 @@ struct lbm_s {
     void *tiles = nullptr;        // tile maxima of the most recent sensor step (one of tilebuf)
     void *tilebuf[2] = {nullptr, nullptr};
     int tile_next = 0;            // buffer the next sensor step writes; it clears the other
+    bool sensor_captured = false; // a caller's graph holds a sensor step: its replays write and clear
+                                  // the buffers they were captured with, so neither is known to be clear
     void *blocks = nullptr;
     double *blocks_f64 = nullptr;
     int8_t *flags = nullptr;
@@ -247,7 +249,14 @@ int ensure_kfield(lbm_t *h) {
 cudaError_t launch_step(lbm_t *h, int src, int mode) {
     StepParams p = params_of(h);
     void *tiles = mode ? h->tilebuf[h->tile_next] : nullptr;
-    if (mode) p.tile_zero = h->tilebuf[h->tile_next ^ 1];
+    if (mode) {
+        p.tile_zero = h->tilebuf[h->tile_next ^ 1];
+        cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+        const cudaError_t e = cudaStreamIsCapturing(h->stream, &capturing);
+        if (e != cudaSuccess) return e;
+        if (capturing != cudaStreamCaptureStatusNone) h->sensor_captured = true;
+        p.tile_clear = !h->sensor_captured;
+    }
     void *kf = (mode == 2) ? h->kfield : nullptr;
     if (h->q == LBM_D2Q9)
         return lbm::step_d2q9(h->dtype, h->buf[src], h->buf[src ^ 1], p, mode, tiles, kf, h->stream,

@@ -487,7 +487,7 @@ inline bool flat_rows(const StepParams &p, int mode, int dtype, int per_lane) {
     if (L::D == 2) return mode == 0 && ragged && dtype == 1 && per_lane == 1;
     if (plane * p.nz < 1LL << 19) return false;
     // a sensor step's tile maxima are combined in a buffer that has to be clear
-    if (mode != 0) return ragged && per_lane == 1 && p.tile_zero;
+    if (mode != 0) return ragged && per_lane == 1 && p.tile_clear;
     return ragged || (per_lane == 2 && p.nx >= 256);
 }
 

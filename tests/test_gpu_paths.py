@@ -334,3 +334,39 @@ def test_2d_steps_of_any_share_of_the_gpu_overlap(L, dtype, nx, ny):  # noqa: F8
         assert np.array_equal(lats[0].sensor(8), lats[1].sensor(8))
     for lat in lats:
         lat.close()
+
+
+@pytest.mark.parametrize("dtype", ["LBM_F32", "LBM_F16S"])
+def test_sensor_steps_replayed_from_a_callers_graph(L, dtype):  # noqa: F811
+    """A plain and a sensor step in a caller's graph, replayed with steps outside it between: each
+    sensor step's maxima are its own, not those of an earlier one in the same buffer."""
+    import torch
+
+    dims = (81, 90, 75)  # ragged rows, over 2^19 cells: a line outside graphs
+    o = O.Oracle(19, *dims, tau=0.7, lid=(0.0, 0.0, 0.0))
+    f = perturbed(o, seed=61, amp=0.05)  # decays from step to step
+    side = torch.cuda.Stream()
+    a, b = [L.Lattice(19, *dims, 0.7, dtype=getattr(L, dtype), lid=(0.0, 0.0), stream=side) for _ in range(2)]
+    for lat in (a, b):
+        lat.set_populations(f)
+        lat.step(2)
+    out = torch.empty(L.lbm_nblocks(a.h, 8), dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        a.step(2)
+        L.lbm_sensor_dev(a.h, 8, out)
+    for k in range(6):
+        if k % 3 == 2:
+            a.step(2)
+            got = a.sensor(8)
+        else:
+            with torch.cuda.stream(side):
+                graph.replay()
+            torch.cuda.synchronize()
+            got = out.cpu().numpy()
+        b.step(2)
+        assert np.array_equal(got, b.sensor(8)), k
+    assert np.array_equal(a.raw(), b.raw())
+    for lat in (a, b):
+        lat.close()
