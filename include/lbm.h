@@ -519,8 +519,10 @@ LBM_API int lbm_blocks_schedule(lbm_t *h, int level, int *form, int *planes, int
  * order.  *nboxes receives the number of boxes; if it exceeds max_boxes, nothing is written to
  * `boxes` and the call returns LBM_EINVAL.  ntagged (may be NULL) receives the number of tag cells
  * tagged after steps 1-3, tags_out (host, tx * ty * tz bytes, may be NULL) the tags themselves
- * (0/1).  Tag, buffer, nesting and the slab counts of each round of boxes run on the GPU; the cut
- * decisions are made on the host between rounds.  Synchronises.  Arguments out of range
+ * (0/1).  All steps run on the GPU, the cut decisions too, except where the tag grid's extents add up
+ * to more than 8192 or a round has more than 8192 boxes (or 2^19 slabs): there the host cuts between
+ * rounds.  Synchronises.  The handle keeps the call's device buffers until lbm_destroy: two bytes a
+ * tag cell of the largest grid so far (four with `allowed`) and about 5 MB.  Arguments out of range
  * (coarsen < 1, buffer < 0, nest < 0, min_width < 1, efficiency outside [0, 1] or NaN) give
  * LBM_EINVAL.
  */

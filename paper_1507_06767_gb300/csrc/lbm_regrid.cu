@@ -270,11 +270,12 @@ int decide(HBox &box, const int *sx, const int *sy, const int *sz, double effici
 // other in the stream without the host.  The CTAs of a launch share the round's boxes evenly: a box
 // is counted by `parts` CTAs, each taking a run of its rows, and the one that comes last decides (no
 // CTA waits for another).  The decisions are those of decide(), over the same integers and the one
-// product of doubles, so the boxes are the same.  A round overlaps its start with the end of the one
-// before, as most rounds of a regrid of few boxes have nothing to do (one box of 128^2 tags: 138 us with
-// plain launches, 121 with the rounds on the host, 94 so; 175 boxes of 64^3 tags 453, 1042, 362).  Of a regrid of 64^3 tags in 12 rounds with its level
+// product of doubles, so the boxes are the same.  Of a regrid of 64^3 tags in 12 rounds with its level
 // map, 732 us, 132 us were kernels, the rest uploads, downloads and waits between the rounds and
-// allocations; with the rounds and the buffers kept on the device it takes 320 us.
+// allocations; with the rounds and the buffers kept on the device it takes 280 us.  A round overlaps its
+// start with the end of the one before, as most rounds of a regrid of few boxes have nothing to do: one
+// box of 128^2 tags takes 90 us, 138 without the overlap and 121 with the rounds on the host; 175 boxes of
+// 64^3 tags 359, 449 and 1042.
 constexpr int CL_THREADS = 256;
 constexpr int CL_CTAS = 608;         // four to an SM
 constexpr int CL_MAX_PARTS = 152;    // CTAs of one box: each adds its x counts to the same few words

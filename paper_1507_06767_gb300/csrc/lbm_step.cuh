@@ -469,15 +469,14 @@ inline cudaError_t launch_step(dim3 grid, dim3 block, cudaStream_t s, Args... ar
 // and the cells a lane takes along x as in the kernels.  Rows that do not fill whole warps leave lanes
 // idle and start anywhere in a memory sector, a line neither (rows -> line, us a plain step: 195 x 129 x
 // 97 FP32 76.3 -> 64.7, FP64 886 -> 773; 250 x 182 x 130 FP32 174 -> 144, BF16 101 -> 95; 100^3 FP16
-// 29.7 -> 22.4; sensor steps of 100^3 FP32 39.2 -> 35.0, of 195 x 129 x
-// 97 FP32 80.9 -> 69.0, FP16 67.4 -> 56.3, BF16 67.0 -> 55.9, of 251 x 181 x 131 FP16 128 -> 122).  Two cells a lane gain in long rows too, as a
-// CTA then reads longer runs (256 x 256 x 128 FP16 124 -> 120, 128 x 128 x 64 unchanged); one cell a lane
+// 29.7 -> 22.4; sensor steps of 100^3 FP32 39.2 -> 35.0, of 195 x 129 x 97 FP32 80.9 -> 69.0, FP16 67.4 ->
+// 56.3, BF16 67.0 -> 55.9, of 251 x 181 x 131 FP16 128 -> 122).  Two cells a lane gain in long rows too, as
+// a CTA then reads longer runs (256 x 256 x 128 FP16 124 -> 120, 128 x 128 x 64 unchanged); one cell a lane
 // does not (256 x 256 x 64 FP32 101.0 -> 100.4), and two lose in sensor steps (250 x 182 x 130 BF16 102
 // -> 105).  Below 2^19 cells the line has fewer than two CTAs an SM, where rows have more and smaller ones
 // (42 x 36 x 227 FP32 18.7 -> 19.8 a sensor step, 40^3 9.8 -> 10.1), except in FP64, which the FP64 units
-// bound (40^3 41 -> 29).  In 2-D
-// FP64 (130^2 6.3 -> 4.9) and FP32 (50 x 700 2.10 -> 1.84, 301 x 203 2.22 -> 2.09) gain, 16-bit types
-// lose (1025 x 1023 10.0 -> 10.5).
+// bound (40^3 41 -> 29).  In 2-D FP64 (130^2 6.3 -> 4.9) and FP32 (50 x 700 2.10 -> 1.84, 301 x 203 2.22 ->
+// 2.09) gain, 16-bit types lose (1025 x 1023 10.0 -> 10.5).
 template <class L>
 inline bool flat_rows(const StepParams &p, int mode, int dtype, int per_lane) {
     const long long plane = (long long)p.nx * p.ny;
