@@ -6,10 +6,11 @@
 // product of segments), the nesting mask (the dual erosion, positions beyond a non-periodic edge
 // counting as covered) and, for every round of candidate boxes, the slab counts (signatures)
 // along each axis.  The cut decisions need only the signatures; the kernel that counts them makes
-// them, or the host between rounds where there are too many boxes for that: shrink to the tags' bounding box, accept at the efficiency, else cut at the hole nearest
-// the centre, else at the strongest inflection of the signature, else bisect the longest axis;
-// cuts leaving a piece narrower than min_width are not admissible.  Boxes of one round are
-// disjoint, so a round costs one pass over at most the tag grid.
+// them, or the host between rounds where there are too many boxes for that: shrink to the tags'
+// bounding box, accept at the efficiency, else cut at the hole nearest the centre, else at the
+// strongest inflection of the signature, else bisect the longest axis; cuts leaving a piece narrower
+// than min_width are not admissible.  Boxes of one round are disjoint, so a round costs one pass over
+// at most the tag grid.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <limits.h>

@@ -475,8 +475,11 @@ inline cudaError_t launch_step(dim3 grid, dim3 block, cudaStream_t s, Args... ar
 // does not (256 x 256 x 64 FP32 101.0 -> 100.4), and two lose in sensor steps (250 x 182 x 130 BF16 102
 // -> 105).  Below 2^19 cells the line has fewer than two CTAs an SM, where rows have more and smaller ones
 // (42 x 36 x 227 FP32 18.7 -> 19.8 a sensor step, 40^3 9.8 -> 10.1), except in FP64, which the FP64 units
-// bound (40^3 41 -> 29).  In 2-D FP64 (130^2 6.3 -> 4.9) and FP32 (50 x 700 2.10 -> 1.84, 301 x 203 2.22 ->
-// 2.09) gain, 16-bit types lose (1025 x 1023 10.0 -> 10.5).
+// bound (40^3 41 -> 29).  Over 47 lattices of odd sides above that line, FP32 and FP16 sensor steps gain
+// 11 %; five of them lose 1 to 5 % in FP32 (151 x 191 x 25 25.1 -> 26.5, 166 x 59 x 99 31.8 -> 32.8), which
+// neither the CTAs an SM nor the lanes saved tell apart from those that gain.  In 2-D FP64 (130^2 6.3 ->
+// 4.9) and FP32 (50 x 700 2.10 -> 1.84, 301 x 203 2.22 -> 2.09) gain, 16-bit types lose (1025 x 1023 10.0 ->
+// 10.5).
 template <class L>
 inline bool flat_rows(const StepParams &p, int mode, int dtype, int per_lane) {
     const long long plane = (long long)p.nx * p.ny;

@@ -61,8 +61,9 @@ __device__ __forceinline__ bool is_finite(double v) {
 //
 // A plain D3Q19 step issues about 165 FP64 instructions a cell (about 350 with each direction relaxed
 // by itself) and takes 0.653 ms at 128^3, 1.081 ms before, with the sensor 1.234 and 1.973; a D2Q9 step at
-// 128^2 4.5 us, 10.9 us before (with the smaller CTAs below).  After 100 steps of a 128^2 cavity the
-// populations are 0.5e-16 to 1.3e-16 off an 80-bit evaluation, 2.2e-16 to 2.7e-16 before.
+// 128^2 4.5 us, 10.9 us before (with the smaller CTAs below).  One warp alone waits for the longer chain of
+// the sensor's sum (4000 x 1 with the sensor at every step 12.4 -> 14.3 us).  After 100 steps of a 128^2
+// cavity the populations are 0.5e-16 to 1.3e-16 off an 80-bit evaluation, 2.2e-16 to 2.7e-16 before.
 template <class L, int MODE, class Emit>
 __device__ __forceinline__ double relax_cell_f64(const double *df, const RelaxF64 &k, bool &mid,
                                                  Emit &&emit) {
